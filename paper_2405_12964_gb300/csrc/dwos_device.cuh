@@ -6,15 +6,14 @@
 //    alpha = P |dB| for the screened Poisson equation (Sec. 3.3.1; G and P are
 //    derived from the PDE because the paper defers them to WoSt App. A)
 //  - closest point on a segment / triangle (DistanceToBoundary, Algorithm 1)
-//  - BVH node layout and a stackless, near-child-first closest-point traversal
-//    over parent links (Hapala et al. 2011 style state machine)
+//  - BVH node layout and the near-child-first closest-point traversal of one lane
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
 namespace dwos {
 
-constexpr int kFromParent = 0x7fffffff;   // traversal state: entered from above
+constexpr int kFromParent = 0x7fffffff;   // inside test's traversal: entered from above
 constexpr int kEmptyChild = 0x7ffffffe;   // child slot with an empty box
 constexpr float kInf = __builtin_inff();
 
@@ -332,49 +331,56 @@ __device__ __forceinline__ bool within(float box_d2, float best2) {
     return box_d2 <= best2 * 1.00001f;
 }
 
+// Traversal stack of one lane, in local memory (held in L1).  A path down the radix
+// tree has at most 62 nodes (30 bits of key, then 32 of index among equal keys) and
+// leaves at most one sibling behind per node.
+constexpr int kLaneStack = 64;
+constexpr int kNoNode = 0x7ffffffd;        // no node or leaf left to visit
+
 // Top-down search of the subtree under internal node `start` for a leaf
-// closer than best2: near-child-first descent; on the way back up each parent
-// is refetched and its children re-ordered by the same box distances, so no
-// stack is needed.  Returns when it climbs back out of `start`.  The budget
-// bounds the node fetches (each node is entered at most three times).
+// closer than best2, near child first; the far child waits on the lane's
+// stack with its distance and is dropped if a closer leaf was found since.
+// (Climbing back over parent links instead fetches each node up to three times,
+// each a dependent round trip to L1 or L2: the bound of a per-lane search.)
+// Lanes first go down to their next leaf, then measure it together.  The
+// budget bounds the node fetches.
 template <int DIM>
 __device__ __forceinline__ bool search_subtree(const BvhView& bvh, int start, const float* q, float& best2, int& best,
                                                int& budget, unsigned& n_nodes, unsigned& n_prims) {
-    int node = start;
-    int from = kFromParent;
+    float2 st[kLaneStack];
+    int sp = 0, cur = start;
     for (;;) {
-        if (--budget < 0) return false;
-        ++n_nodes;
-        float lo0[DIM], hi0[DIM], lo1[DIM], hi1[DIM];
-        int c0, c1, parent;
-        load_node<DIM>(bvh.nodes, node, lo0, hi0, lo1, hi1, c0, c1, parent);
-        const float d0 = box_dist2<DIM>(q, lo0, hi0);
-        const float d1 = box_dist2<DIM>(q, lo1, hi1);
-        const bool first0 = d0 <= d1;
-        const int nearc = first0 ? c0 : c1, farc = first0 ? c1 : c0;
-        const float dn = first0 ? d0 : d1, df = first0 ? d1 : d0;
-        int state = (from == kFromParent) ? 0 : (from == nearc ? 1 : 2);
-        int next = kFromParent;
-        for (;;) {
-            int cand = kFromParent;
-            if (state == 0) { if (within(dn, best2)) cand = nearc; else state = 2; }
-            if (state == 1) { if (within(df, best2)) cand = farc; }
-            if (cand == kFromParent) break;
-            if (cand < 0) {                       // leaf: test in place
-                const int p = ~cand;
-                ++n_prims;
-                const float dd = prim_dist2<DIM>(bvh.prims, p, q);
-                if (closer(dd, p, best2, best)) { best2 = dd; best = p; }
-                state = (state == 0) ? 1 : 2;
-                continue;
+        while (cur >= 0 && cur != kNoNode) {
+            if (--budget < 0) return false;
+            ++n_nodes;
+            float lo0[DIM], hi0[DIM], lo1[DIM], hi1[DIM];
+            int c0, c1, parent;
+            load_node<DIM>(bvh.nodes, cur, lo0, hi0, lo1, hi1, c0, c1, parent);
+            const float d0 = box_dist2<DIM>(q, lo0, hi0);
+            const float d1 = box_dist2<DIM>(q, lo1, hi1);
+            const bool first0 = d0 <= d1;
+            const int nearc = first0 ? c0 : c1, farc = first0 ? c1 : c0;
+            const float dn = first0 ? d0 : d1, df = first0 ? d1 : d0;
+            if (farc != kEmptyChild && within(df, best2)) {
+                if (sp >= kLaneStack) return false;
+                st[sp++] = make_float2(df, __int_as_float(farc));
             }
-            next = cand;
-            break;
+            cur = nearc != kEmptyChild && within(dn, best2) ? nearc : kNoNode;
+            while (cur == kNoNode && sp > 0) {
+                const float2 e = st[--sp];
+                if (within(e.x, best2)) cur = __float_as_int(e.y);
+            }
         }
-        if (next != kFromParent) { from = kFromParent; node = next; continue; }
-        if (node == start) return true;
-        from = node;
-        node = parent;
+        if (cur == kNoNode) return true;
+        const int p = ~cur;
+        ++n_prims;
+        const float dd = prim_dist2<DIM>(bvh.prims, p, q);
+        if (closer(dd, p, best2, best)) { best2 = dd; best = p; }
+        cur = kNoNode;
+        while (cur == kNoNode && sp > 0) {
+            const float2 e = st[--sp];
+            if (within(e.x, best2)) cur = __float_as_int(e.y);
+        }
     }
 }
 
