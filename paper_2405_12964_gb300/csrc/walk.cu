@@ -29,10 +29,13 @@ constexpr unsigned kFull = 0xffffffffu;
 // Search order 3 routes each query by the binary root's two child boxes: most
 // queries (closer to an outsized element, or to their seed, than to any tree
 // box) need no tree search at all; the few that do are searched by the whole
-// warp over the 32-wide tree, one at a time, unless more than this many lanes
-// of the warp need one in the same step, when each searches the binary tree.
-constexpr int kRouteWideMax2 = 16;   // segments
-constexpr int kRouteWideMax3 = 32;   // triangles: the per-lane binary search never pays
+// warp over the 32-wide tree, one at a time.  Segments are searched one query per
+// lane, over the binary tree, where more than kLaneSearchMin lanes of the warp need
+// a search in the same step (16 or 33: within 2 % on a 4096-segment star whose
+// points' queries mostly need one) or the tree has at most kLaneTreeMax leaves (128
+// segments: 0.34 ms against 0.42 ms by groups of lanes); triangles never.
+constexpr int kLaneSearchMin = 16;
+constexpr int kLaneTreeMax = 256;
 
 template <int DIM>
 __device__ __forceinline__ float field_value(const float* c, const float* x, float* grad) {
@@ -128,7 +131,7 @@ __device__ __forceinline__ void sphere_dir(const U4& r, float* om) {
 template <int DIM, bool WIDE, bool STAR = false, bool CONES = false, bool DATA = false>
 __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
     walk_kernel(const DevProblem* __restrict__ g_probs, int n_probs, unsigned long long total,
-                DevCounters* __restrict__ ctr, DevCounters* __restrict__ zero_ctr,
+                DevCounters* __restrict__ ctr, DevCounters* __restrict__ zero_ctr, int lanes,
                 const __grid_constant__ DevProblem p_arg) {
     constexpr bool wide = WIDE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -169,7 +172,7 @@ __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
     for (int k = 0; k < DIM; ++k) { n_on[k] = 0.0f; n2[k] = 0.0f; }
 
     const int lane = threadIdx.x & 31;
-    bool active = false, exhausted = false;
+    bool active = false, exhausted = lane >= lanes;
     int error = 0;
     WarpStats st;
 
@@ -262,9 +265,9 @@ __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
                     }
                 }
                 need = __ballot_sync(kFull, desc);
-                if (__popc(need) > (DIM == 2 ? kRouteWideMax2 : kRouteWideMax3)) {   // many searches this step: one per lane, in parallel
-                    lane_search = desc;
-                    need = 0;
+                if (DIM == 2) {
+                    lane_search = desc && (Pw.n_tree <= kLaneTreeMax || __popc(need) > kLaneSearchMin);
+                    need = __ballot_sync(kFull, desc && !lane_search);
                 }
             }
             if (need) {   // all lanes search the 32-wide tree together, one lane's query at a time
@@ -825,16 +828,24 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
         return cudaSuccess;
     }
     const int bs = L.block_size;
+    if (bs % 32 != 0) return cudaErrorInvalidValue;
     if (L.star && n_probs != 1) return cudaErrorInvalidValue;
     int per_sm = L.blocks_per_sm > 0 ? L.blocks_per_sm
                                      : walk_max_blocks_per_sm(L.dim, bs, L.traversal, L.star, L.cones, L.data);
     if (per_sm < 1) per_sm = 1;
+    // A launch that cannot fill every lane spreads its walks over all warps, a few lanes
+    // each: a warp's iteration lasts as long as its lanes' searches take in turn, and the
+    // launch as long as its longest walks.  Walk kernel of 512 walks over a 4096-segment
+    // star 0.68 ms with full warps, 0.14 ms with one walk per warp; 3,200 walks over 5,800
+    // triangles 2.5 -> 0.46 ms; 8 points x 300 walks over 777 segments 0.75 -> 0.12 ms.
+    const unsigned long long warps = (unsigned long long)per_sm * L.n_sm * (bs / 32);
+    const int lanes = total < 32 * warps ? (int)((total + warps - 1) / warps) : 32;
+    const unsigned long long per_block = (unsigned long long)lanes * (bs / 32);
     long long blocks = (long long)per_sm * L.n_sm;
-    const long long need = (long long)((total + bs - 1) / bs);
+    const long long need = (long long)((total + per_block - 1) / per_block);
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     if (blocks_used) *blocks_used = (int)blocks;
-    if (bs % 32 != 0) return cudaErrorInvalidValue;
     const size_t smem = walk_smem_bytes(n_probs, bs, L.traversal, L.dim, L.star);
     DevProblem P1;
     if (host_prob) P1 = *host_prob;
@@ -844,7 +855,7 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kernel<<<(int)blocks, bs, smem, stream>>>(d_probs, n_probs, total, d_counters, zero_counters, P1);
+        kernel<<<(int)blocks, bs, smem, stream>>>(d_probs, n_probs, total, d_counters, zero_counters, lanes, P1);
         return cudaGetLastError();
     };
     if (L.star) {
