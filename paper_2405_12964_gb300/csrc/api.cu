@@ -480,6 +480,7 @@ dwos_status run_walks(dwos_ctx* ctx, int n_query, const float* xq, int W, unsign
     L.blocks_per_sm = ctx->opt.blocks_per_sm;
     L.n_sm = ctx->n_sm;
     L.traversal = P.traversal;
+    L.wide_depth = ctx->bvh.wide_depth;
     L.star = P.neu != nullptr;
     L.cones = L.star && ctx->neu_host.sil_cone_node != nullptr;
     L.data = L.star && ctx->neu_host.flux != nullptr;
@@ -1314,7 +1315,7 @@ dwos_status dwos_bvh_info(const dwos_ctx* ctx, int32_t* info) {
     info[1] = ctx->bvh.n_tree;
     info[2] = ctx->bvh.n_big;
     info[3] = ctx->bvh.n_internal;
-    info[4] = ctx->bvh.n_wide;
+    info[4] = (int32_t)wide_units(ctx->dim, ctx->bvh.n_wide);
     info[5] = ctx->bvh.wide_depth;
     return DWOS_OK;
 }
@@ -1409,7 +1410,7 @@ dwos_status dwos_last_stats(dwos_ctx* ctx, dwos_run_stats* out) {
     out->capped = c.capped;
     out->nodes_visited = c.nodes;
     out->prims_tested = c.prims;
-    out->wide_nodes_visited = c.wnodes;
+    out->wide_nodes_visited = wide_units(ctx->dim, c.wnodes);
     out->launches = ctx->launches;
     out->blocks = ctx->last_blocks;
     float ms = 0.0f;
@@ -1706,6 +1707,7 @@ extern "C" dwos_status dwos_eval_static(dwos_ctx* ctx, int n_query, const float*
     L.blocks_per_sm = ctx->opt.blocks_per_sm;
     L.n_sm = ctx->n_sm;
     L.traversal = P.traversal;
+    L.wide_depth = ctx->bvh.wide_depth;
     int blocks = 0;
     CK(launch_walks(L, d_prob, 1, total, d_ctr, ctx->stream, &blocks), "walk kernel");
     CK(launch_reduce_u(d_rec, n_query, W, u_mean, u_se, ctx->stream), "reduce u");

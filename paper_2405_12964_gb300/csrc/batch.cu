@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "ctx.h"
+#include "dwos_device.cuh"
 #include "dwos_internal.h"
 
 using namespace dwos;
@@ -253,8 +254,10 @@ dwos_status dwos_batch_create(dwos_batch** out, const dwos_batch_job* jobs, int 
         }
         b->cfg[dim].dim = dim;
         b->cfg[dim].block_size = 256;
-        b->cfg[dim].blocks_per_sm = std::max(1, walk_max_blocks_per_sm(dim, 256));
+        b->cfg[dim].blocks_per_sm = std::max(1, walk_max_blocks_per_sm(b->cfg[dim]));
         b->cfg[dim].n_sm = b->n_sm;
+        // (two levels to spare: a context may rebuild its tree after the batch was made)
+        for (int ji : ids) b->cfg[dim].wide_depth = std::max(b->cfg[dim].wide_depth, b->jobs[ji].ctx->bvh.wide_depth + 2);
     }
     if (dwos_status s = upload_tables(b)) return bail(s);
     if ((e = cudaEventCreate(&b->ev0)) != cudaSuccess || (e = cudaEventCreate(&b->ev1)) != cudaSuccess)
@@ -348,7 +351,10 @@ dwos_status dwos_batch_autotune(dwos_batch* b, int reps) {
             b->trav[dim] = trav;
             if (dwos_status s = upload_tables(b)) return s;
             for (int bs : sizes) {
-                const int maxb = std::max(1, walk_max_blocks_per_sm(dim, bs, trav));
+                WalkLaunch probe = b->cfg[dim];
+                probe.block_size = bs;
+                probe.traversal = trav;
+                const int maxb = std::max(1, walk_max_blocks_per_sm(probe));
                 for (int per = 1; per <= maxb; per = per < maxb ? std::min(maxb, per * 2) : maxb + 1) {
                     WalkLaunch L = b->cfg[dim];
                     L.block_size = bs;
@@ -444,7 +450,7 @@ dwos_status dwos_batch_stats(dwos_batch* b, dwos_run_stats* out) {
         out->capped += c.capped;
         out->nodes_visited += c.nodes;
         out->prims_tested += c.prims;
-        out->wide_nodes_visited += c.wnodes;
+        out->wide_nodes_visited += wide_units(ch.dim, c.wnodes);
         if (c.error & 4) return bfail(b, DWOS_ERR_INVALID_ARG, "a query point is not finite");
         if (c.error & 1) return bfail(b, DWOS_ERR_STEP_LIMIT, "BVH traversal exceeded its iteration bound");
     }

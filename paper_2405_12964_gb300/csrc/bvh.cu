@@ -2,15 +2,12 @@
 //   element boxes + scene bounds -> Morton codes -> radix sort (CUB) ->
 //   binary radix tree (Karras, "Maximizing parallelism in the construction of
 //   BVHs, octrees and k-d trees", HPG 2012) -> bottom-up box refit with
-//   arrival counters -> leaf primitives written in Morton order -> 32-wide
-//   tree collapsed from the binary one five levels at a time.
+//   arrival counters -> leaf primitives written in Morton order -> wide tree
+//   collapsed from the binary one (2D: 32 axis-aligned slots, 3D: 8 oriented ones).
 // Plus the batched closest-point, ray-parity inside test and Philox kernels.
 #include <cub/device/device_radix_sort.cuh>
-#include <cub/device/device_scan.cuh>
 
 #include <cstring>
-#include <utility>
-#include <vector>
 
 #include "dwos_device.cuh"
 #include "dwos_internal.h"
@@ -337,24 +334,22 @@ __global__ void single_leaf_kernel(const float* vert, const int* elem, const int
         make_float4(__int_as_float(~0), __int_as_float(kEmptyChild), __int_as_float(-1), 0.0f);
 }
 
-// ---- 32-wide tree -----------------------------------------------------------
+// ---- wide tree --------------------------------------------------------------
 // Built top-down, one level per launch.  A wide node starts from its binary
 // root's two children; it first opens, largest first, the inner children with
-// more than 32 leaves (they cannot become one leaf-level node), then absorbs
+// more than W leaves (they cannot become one leaf-level node), then absorbs
 // whole inner children that still fit as their leaves, largest first.  Its
 // remaining inner children become the next level's wide nodes.  (Opening
 // every child by size alone cuts small subtrees into pieces, each a nearly
-// empty wide node: 37 % of the slots used on a 32 k-element test set against
+// empty wide node: 37 % of 32 slots used on a 32 k-element test set against
 // 71 % with this rule.)
 
-// Frontier of each wide node of this level (in order), and its inner-child count.
-__global__ void wide_level_kernel(const int* node_child, const int* node_count, const int* node_first,
-                                  const int* leaf_parent, const int* roots, int m, int* fr_code, int* fr_src,
-                                  int* n_inner) {
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= m) return;
-    const int r = roots[w];
-    int code[kWide], src[kWide];
+// The children of the wide node whose binary root is r: their codes (>= 0: binary
+// node, < 0: ~leaf) and the binary tree's slots of their boxes ((parent << 1) |
+// side); returns their number.
+template <int W>
+__device__ __forceinline__ int wide_children(const int* node_child, const int* node_count, const int* node_first,
+                                             const int* leaf_parent, int r, int* code, int* src) {
     int cnt = 0;
     for (int side = 0; side < 2; ++side) {
         code[cnt] = node_child[2 * r + side];
@@ -362,8 +357,8 @@ __global__ void wide_level_kernel(const int* node_child, const int* node_count, 
         ++cnt;
     }
     auto leaves = [&](int c) { return c >= 0 ? node_count[c] : 1; };
-    while (cnt < kWide) {                      // open the largest child with more than 32 leaves
-        int pick = -1, best = kWide;
+    while (cnt < W) {                          // open the largest child with more than W leaves
+        int pick = -1, best = W;
         for (int i = 0; i < cnt; ++i)
             if (code[i] >= 0 && leaves(code[i]) > best) { best = leaves(code[i]); pick = i; }
         if (pick < 0) break;
@@ -375,8 +370,8 @@ __global__ void wide_level_kernel(const int* node_child, const int* node_count, 
         }
         ++cnt;
     }
-    while (cnt < kWide) {                      // absorb the largest inner child that fits
-        const int room = kWide - cnt + 1;
+    while (cnt < W) {                          // absorb the largest inner child that fits
+        const int room = W - cnt + 1;
         int pick = -1, best = 0;
         for (int i = 0; i < cnt; ++i)
             if (code[i] >= 0 && leaves(code[i]) <= room && leaves(code[i]) > best) { best = leaves(code[i]); pick = i; }
@@ -390,33 +385,51 @@ __global__ void wide_level_kernel(const int* node_child, const int* node_count, 
         }
         cnt += k - 1;
     }
-    int inner = 0;
-    for (int i = 0; i < kWide; ++i) {
-        const bool used = i < cnt;
-        fr_code[kWide * w + i] = used ? code[i] : kEmptyChild;
-        fr_src[kWide * w + i] = used ? src[i] : -1;
-        inner += (used && code[i] >= 0) ? 1 : 0;
-    }
-    n_inner[w] = inner;
+    return cnt;
 }
 
-// Wide-node codes of the inner children (the next level, numbered after
-// next_base in order) and the next level's binary roots.
-__global__ void wide_assign_kernel(const int* fr_code, const int* fr_src, const int* offset, int m, int next_base,
-                                   int* wcode, int* wsrc, int* next_roots) {
+// lev[L]: wide nodes of level L.  A level's kernel reads its own count, which the
+// kernel before it finished, so the host enqueues every level without waiting
+// and reads the counts once (a copy, a wait and six allocations per level took
+// longer than the levels themselves).  Per wide node: its binary root and its first
+// inner child's id (the inner children of a node have consecutive ids).  Ids are
+// given out by an atomic counter: a node's number varies from build to build, its
+// children and their order do not.
+template <int W>
+__global__ void wide_level_kernel(const int* node_child, const int* node_count, const int* node_first,
+                                  const int* leaf_parent, int level, int* lev, int* wroot, int* wnext) {
+    int base = 0;
+    for (int l = 0; l < level; ++l) base += lev[l];
+    const int m = lev[level];
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x) {
+        int code[W], src[W];
+        const int cnt = wide_children<W>(node_child, node_count, node_first, leaf_parent, wroot[base + i], code, src);
+        int inner = 0;
+        for (int k = 0; k < cnt; ++k) inner += code[k] >= 0 ? 1 : 0;
+        int id = base + m + (inner ? atomicAdd(lev + level + 1, inner) : 0);
+        wnext[base + i] = id;
+        for (int k = 0; k < cnt; ++k)
+            if (code[k] >= 0) wroot[id++] = code[k];
+    }
+}
+
+// Per slot: the child's code in the wide tree and the binary tree's slot of its box (-1:
+// unused); per wide node, the slot that holds it.
+template <int W>
+__global__ void wide_codes_kernel(const int* node_child, const int* node_count, const int* node_first,
+                                  const int* leaf_parent, int n_wide, const int* wroot, const int* wnext, int* wcode,
+                                  int* wsrc, int* wslot) {
     const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= m) return;
-    int k = offset[w];
-    for (int i = 0; i < kWide; ++i) {
-        const int c = fr_code[kWide * w + i];
-        wsrc[kWide * w + i] = fr_src[kWide * w + i];
-        if (c >= 0 && c != kEmptyChild) {
-            next_roots[k] = c;
-            wcode[kWide * w + i] = next_base + k;
-            ++k;
-        } else {
-            wcode[kWide * w + i] = c;
-        }
+    if (w >= n_wide) return;
+    int code[W], src[W];
+    const int cnt = wide_children<W>(node_child, node_count, node_first, leaf_parent, wroot[w], code, src);
+    int id = wnext[w];
+    if (w == 0) wslot[0] = -1;
+    for (int k = 0; k < W; ++k) {
+        const bool in = k < cnt && code[k] >= 0;
+        wsrc[W * w + k] = k < cnt ? src[k] : -1;
+        if (in) wslot[id] = W * w + k;
+        wcode[W * w + k] = in ? id++ : (k < cnt ? code[k] : kEmptyChild);
     }
 }
 
@@ -464,6 +477,199 @@ __global__ void wide_refit_kernel(const float4* nodes, const float4* prims, cons
     for (int k = 0; k < DIM * DIM; ++k) f[WideLayout<DIM>::kVtx + k * kWide + j] = v[k];
 }
 
+__device__ __forceinline__ float warp_fsum(float v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ float warp_fmin(float v) {
+    for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+__device__ __forceinline__ float warp_fmax(float v) { return -warp_fmin(-v); }
+
+// Up to this many leaves a node gets a box oriented by its elements' mean normal;
+// above it the axis-aligned box of the binary tree (a patch that large is curved, and
+// the pass over its leaves would dominate the refit: 15.2 visits per query with a limit
+// of 1024, 15.7 without one, 18.8 with one of 64, on the 200k-triangle sphere).
+constexpr int kOrientMax = 512;
+
+// Vertex a of triangle leaf p.
+__device__ __forceinline__ void leaf_vertex(const float4* prims, int p, int a, float* v) {
+    const float4 s = __ldg(prims + 3 * p + a);
+    v[0] = s.x; v[1] = s.y; v[2] = s.z;
+}
+
+// Its normal, of twice its area's length.
+__device__ __forceinline__ void leaf_normal(const float4* prims, int p, float* n) {
+    float a[3], b[3], c[3];
+    leaf_vertex(prims, p, 0, a);
+    leaf_vertex(prims, p, 1, b);
+    leaf_vertex(prims, p, 2, c);
+    const float u[3] = {b[0] - a[0], b[1] - a[1], b[2] - a[2]};
+    const float v[3] = {c[0] - a[0], c[1] - a[1], c[2] - a[2]};
+    n[0] = u[1] * v[2] - u[2] * v[1];
+    n[1] = u[2] * v[0] - u[0] * v[2];
+    n[2] = u[0] * v[1] - u[1] * v[0];
+}
+
+// The frame of the unit normal n (row 0) and the unit tangent t (row 1).
+__device__ __forceinline__ void frame_rows(const float* n, const float* t, float (*R)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) { R[0][k] = n[k]; R[1][k] = t[k]; }
+    R[2][0] = n[1] * t[2] - n[2] * t[1];
+    R[2][1] = n[2] * t[0] - n[0] * t[2];
+    R[2][2] = n[0] * t[1] - n[1] * t[0];
+}
+
+// Row r of a frame times (v - o), in the order of the search's box test.
+__device__ __forceinline__ float along(const float* r, const float* v, const float* o) {
+    return fmaf(r[0], v[0] - o[0], fmaf(r[1], v[1] - o[1], r[2] * (v[2] - o[2])));
+}
+
+// Box slot `slot` (node * kOriented + j): centre c, rows R, half extents h with the
+// margin for the rounding of the search's box test (2e-6 of the largest), the code.
+__device__ __forceinline__ void store_box(float4* wnodes, int slot, const float* c, const float (*R)[3],
+                                          const float* h, int code) {
+    const float m = 2e-6f * fmaxf(h[0], fmaxf(h[1], h[2]));
+    float4* o = wnodes + (size_t)(slot / kOriented) * kOrientedF4 + slot % kOriented;
+    o[0] = make_float4(c[0], c[1], c[2], __int_as_float(code));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) o[(1 + k) * kOriented] = make_float4(R[k][0], R[k][1], R[k][2], h[k] + m);
+}
+
+// The oriented boxes of a 3D tree, one warp per wide node: the node's own box, in its
+// parent's slot, and the boxes of its leaf children and empty slots, one per lane.  A
+// box's frame is the mean normal of the elements under it (each counted along the
+// first one's side; a leaf's own normal and first edge); its extents are taken about
+// its rounded centre, so that only relative rounding is left.
+__global__ void oriented_fill_kernel(const float4* nodes, const float4* prims, const int* node_count,
+                                     const int* node_first, const int* wcode, const int* wroot, const int* wslot,
+                                     int n_wide, float4* wnodes) {
+    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (w >= n_wide) return;                      // whole warps exit together
+    const int my_code = lane < kOriented ? wcode[kOriented * w + lane] : 0;
+    if (lane < kOriented && (my_code < 0 || my_code == kEmptyChild)) {
+        float c[3] = {0.0f, 0.0f, 0.0f}, h[3] = {0.0f, 0.0f, 0.0f};
+        float R[3][3] = {{1.0f, 0.0f, 0.0f}, {0.0f, 1.0f, 0.0f}, {0.0f, 0.0f, 1.0f}};
+        if (my_code < 0) {
+            float v[3][3], n[3], t[3], l2 = 0.0f, t2 = 0.0f;
+            for (int a = 0; a < 3; ++a) leaf_vertex(prims, ~my_code, a, v[a]);
+            leaf_normal(prims, ~my_code, n);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                t[k] = v[1][k] - v[0][k];
+                l2 = fmaf(n[k], n[k], l2);
+                t2 = fmaf(t[k], t[k], t2);
+            }
+            const float len = sqrtf(l2), tlen = sqrtf(t2);
+            if (len > 0.0f && len < kInf && tlen > 0.0f && tlen < kInf) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) { n[k] /= len; t[k] /= tlen; }
+                frame_rows(n, t, R);
+            }
+            float m[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                float lo = kInf, hi = -kInf;
+                for (int a = 0; a < 3; ++a) {
+                    const float y = along(R[k], v[a], v[0]);
+                    lo = fminf(lo, y);
+                    hi = fmaxf(hi, y);
+                }
+                m[k] = 0.5f * (lo + hi);
+            }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) c[i] = v[0][i] + (R[0][i] * m[0] + R[1][i] * m[1] + R[2][i] * m[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                for (int a = 0; a < 3; ++a) h[k] = fmaxf(h[k], fabsf(along(R[k], v[a], c)));
+        }
+        store_box(wnodes, kOriented * w + lane, c, R, h, my_code);
+    }
+    const int slot = wslot[w];
+    if (slot < 0) return;                         // the root is in no slot
+    const int b = wroot[w], cnt = node_count[b], first = node_first[b];
+    float R[3][3] = {{1.0f, 0.0f, 0.0f}, {0.0f, 1.0f, 0.0f}, {0.0f, 0.0f, 1.0f}};
+    float c[3], h[3];
+    {                                             // axis-aligned frame and box
+        float lo0[3], hi0[3], lo1[3], hi1[3];
+        int c0, c1, parent;
+        load_node<3>(nodes, b, lo0, hi0, lo1, hi1, c0, c1, parent);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float lo = fminf(lo0[k], lo1[k]), hi = fmaxf(hi0[k], hi1[k]);
+            c[k] = 0.5f * (lo + hi);
+            h[k] = fmaxf(hi - c[k], c[k] - lo);
+        }
+    }
+    if (cnt <= kOrientMax) {
+        float ref[3], n[3] = {0.0f, 0.0f, 0.0f}, area = 0.0f;
+        leaf_normal(prims, first, ref);
+#pragma unroll 4
+        for (int p = first + lane; p < first + cnt; p += 32) {
+            float m[3];
+            leaf_normal(prims, p, m);
+            const float d = m[0] * ref[0] + m[1] * ref[1] + m[2] * ref[2];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) n[k] += d < 0.0f ? -m[k] : m[k];
+            area += sqrtf(m[0] * m[0] + m[1] * m[1] + m[2] * m[2]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n[k] = warp_fsum(n[k]);
+        area = warp_fsum(area);
+        const float len = sqrtf(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+        // a patch whose normals spread too far keeps the axis-aligned box
+        if (len > 0.7f * area && len > 0.0f && area < kInf) {
+            float t[3], o[3], lo[3], hi[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) n[k] /= len;
+            // the axis least aligned with n gives the tangent
+            const float ax = fabsf(n[0]), ay = fabsf(n[1]), az = fabsf(n[2]);
+            if (ax <= ay && ax <= az) { t[0] = 0.0f; t[1] = n[2]; t[2] = -n[1]; }
+            else if (ay <= az) { t[0] = -n[2]; t[1] = 0.0f; t[2] = n[0]; }
+            else { t[0] = n[1]; t[1] = -n[0]; t[2] = 0.0f; }
+            const float il = rsqrtf(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) t[k] *= il;
+            frame_rows(n, t, R);
+            leaf_vertex(prims, first, 0, o);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { lo[k] = kInf; hi[k] = -kInf; }
+#pragma unroll 2
+            for (int p = first + lane; p < first + cnt; p += 32)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    float v[3];
+                    leaf_vertex(prims, p, a, v);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const float y = along(R[k], v, o);
+                        lo[k] = fminf(lo[k], y);
+                        hi[k] = fmaxf(hi[k], y);
+                    }
+                }
+            float m[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { m[k] = 0.5f * (warp_fmin(lo[k]) + warp_fmax(hi[k])); h[k] = 0.0f; }
+#pragma unroll
+            for (int i = 0; i < 3; ++i) c[i] = o[i] + (R[0][i] * m[0] + R[1][i] * m[1] + R[2][i] * m[2]);
+#pragma unroll 2
+            for (int p = first + lane; p < first + cnt; p += 32)
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    float v[3];
+                    leaf_vertex(prims, p, a, v);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) h[k] = fmaxf(h[k], fabsf(along(R[k], v, c)));
+                }
+#pragma unroll
+            for (int k = 0; k < 3; ++k) h[k] = warp_fmax(h[k]);
+        }
+    }
+    if (lane == 0) store_box(wnodes, slot, c, R, h, w);
+}
+
 // ---- queries --------------------------------------------------------------
 template <int DIM>
 __global__ void closest_kernel(BvhView bvh, const int* prim_elem, const int* leaf_of_elem, int n, const float* p,
@@ -506,14 +712,14 @@ __global__ void closest_kernel(BvhView bvh, const int* prim_elem, const int* lea
     bary[2 * i + 1] = w2;
 }
 
-// The same query with the warp-wide search of the 32-wide tree: all lanes of a
+// The same query with the warp's search of the wide tree: all lanes of a
 // block take part (a lane past n only helps), so there is no early return.
 template <int DIM>
 __global__ void closest_wide_kernel(BvhView bvh, WideView wv, const int* prim_elem, const int* leaf_of_elem, int n,
                                     const float* p, const int* hint_elem, float* dist, int* elem_out, float* bary,
-                                    int* err, DevCounters* ctr) {
+                                    int* err, DevCounters* ctr, int stk_cap) {
     extern __shared__ float2 wide_stack[];
-    float2* stk = wide_stack + (size_t)(threadIdx.x >> 5) * kWideStack;
+    float2* stk = wide_stack + (size_t)(threadIdx.x >> 5) * (wide_smem_bytes(DIM, stk_cap) / sizeof(float2));
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const bool act = i < n;
     float q[DIM];
@@ -532,7 +738,7 @@ __global__ void closest_wide_kernel(BvhView bvh, WideView wv, const int* prim_el
         }
         big_closest<DIM>(bvh.prims, bvh.n_tree, bvh.n_big, q, best2, best, np);
     }
-    const int e = wide_closest<DIM>(wv, __ballot_sync(kWarpAll, act), q, best2, best, stk, nn, np);
+    const int e = wide_search<DIM>(wv, __ballot_sync(kWarpAll, act), q, best2, best, stk, stk_cap, nn, np);
     if (e) atomicOr(err, 1);
     if (ctr) {
         atomicAdd(&ctr->wnodes, (unsigned long long)nn);
@@ -768,6 +974,8 @@ inline int nblk(long long n, int b) { return (int)((n + b - 1) / b); }
 
 }  // namespace
 
+constexpr int kWideLevels = 16;   // level counts kept by a wide tree's build
+
 cudaError_t bvh_reserve(BvhBuffers& b, int dim, int n_elem) {
     if (n_elem <= b.capacity && dim == b.dim) return cudaSuccess;
     bvh_free(b);
@@ -789,6 +997,8 @@ cudaError_t bvh_reserve(BvhBuffers& b, int dim, int n_elem) {
     DW_TRY(cudaMalloc(&b.counters, sizeof(int) * (size_t)n_int));
     DW_TRY(cudaMalloc(&b.node_count, sizeof(int) * 2 * (size_t)n_int));   // leaf counts, then first leaves
     DW_TRY(cudaMalloc(&b.node_cell, sizeof(float) * 2 * dim * (size_t)n_int));
+    DW_TRY(cudaMalloc(&b.wroot, sizeof(int) * 2 * (size_t)n_int));        // roots, then first inner children
+    DW_TRY(cudaMalloc(&b.wlev, sizeof(int) * kWideLevels));
     DW_TRY(cudaMalloc(&b.bounds, sizeof(unsigned int) * 6));
     DW_TRY(cudaMalloc(&b.stats, sizeof(float) * 2 + sizeof(int) * 4));
     size_t tmp = 0;
@@ -806,98 +1016,72 @@ void bvh_free(BvhBuffers& b) {
     cudaFree(b.vals); cudaFree(b.vals_sorted); cudaFree(b.leaf_parent); cudaFree(b.node_parent);
     cudaFree(b.node_child); cudaFree(b.counters); cudaFree(b.bounds); cudaFree(b.stats); cudaFree(b.node_cell);
     cudaFree(b.sort_tmp);
-    cudaFree(b.wnodes); cudaFree(b.wsrc); cudaFree(b.node_count);
+    cudaFree(b.wnodes); cudaFree(b.wsrc); cudaFree(b.wroot); cudaFree(b.wlev); cudaFree(b.node_count);
     b = BvhBuffers();
 }
 
 constexpr int kMaxBig = 64;
 
+// The wide tree's boxes (and, in 2D, leaf children's vertices) from the binary tree.
+template <int DIM>
+static cudaError_t fill_wide(BvhBuffers& b, cudaStream_t s) {
+    if constexpr (DIM == 2) {
+        wide_refit_kernel<DIM><<<nblk((long long)b.n_wide * kWide, 256), 256, 0, s>>>(
+            b.nodes, b.prims, b.wsrc, b.wsrc + kWide * (size_t)b.n_wide, b.n_wide, b.wnodes);
+    } else {
+        oriented_fill_kernel<<<nblk(32LL * b.n_wide, 128), 128, 0, s>>>(
+            b.nodes, b.prims, b.node_count, b.node_count + b.n_internal, b.wsrc + kOriented * (size_t)b.n_wide,
+            b.wroot, b.wsrc + 2 * kOriented * (size_t)b.n_wide, b.n_wide, reinterpret_cast<float4*>(b.wnodes));
+    }
+    return cudaGetLastError();
+}
+
 // Collapse the binary tree (n_internal >= 1 nodes, boxes refit) into the
-// 32-wide tree, level by level (one host synchronisation per level reads the
-// next level's size).  Nodes are numbered in level order, the root first.
+// wide tree.  Nodes are numbered level by level, the root first.
 template <int DIM>
 static cudaError_t build_wide(BvhBuffers& b, cudaStream_t s) {
+    constexpr int W = DIM == 2 ? kWide : kOriented;
+    constexpr int kNodeFloats = DIM == 2 ? WideLayout<2>::kFloats : 4 * kOrientedF4;
+    constexpr int kMax = DIM == 2 ? (kWideStack - 1) / (kWide - 1) : kOrientedDepthMax;   // levels the search takes
+    static_assert(kMax < kWideLevels, "level counts");
     const int n_int = b.n_internal;
-    cudaError_t e = cudaSuccess;
-    std::vector<int*> lv_code, lv_src;      // per level: final codes and sources of its nodes
-    std::vector<int> lv_m;
-    int* roots = nullptr;
-    int* next = nullptr;
-    int* fr_code = nullptr;
-    int* fr_src = nullptr;
-    int* n_inner = nullptr;
-    int* offset = nullptr;
-    int m = 1, base = 0, depth = 0;
-    auto cleanup = [&]() {
-        for (int* p : lv_code) cudaFree(p);
-        for (int* p : lv_src) cudaFree(p);
-        cudaFree(roots); cudaFree(next); cudaFree(fr_code); cudaFree(fr_src); cudaFree(n_inner); cudaFree(offset);
-    };
-#define DW_W(x) do { e = (x); if (e != cudaSuccess) { cleanup(); return e; } } while (0)
-    DW_W(cudaMalloc(&roots, sizeof(int)));
-    DW_W(cudaMemsetAsync(roots, 0, sizeof(int), s));          // the binary root is node 0
-    while (m > 0) {
-        if (++depth > 64) { cleanup(); return cudaErrorInvalidValue; }   // a 64-level wide tree cannot happen
-        int *lc = nullptr, *ls = nullptr;
-        DW_W(cudaMalloc(&lc, sizeof(int) * kWide * (size_t)m));
-        lv_code.push_back(lc);
-        DW_W(cudaMalloc(&ls, sizeof(int) * kWide * (size_t)m));
-        lv_src.push_back(ls);
-        lv_m.push_back(m);
-        cudaFree(fr_code); cudaFree(fr_src); cudaFree(n_inner); cudaFree(offset);
-        fr_code = fr_src = n_inner = offset = nullptr;
-        DW_W(cudaMalloc(&fr_code, sizeof(int) * kWide * (size_t)m));
-        DW_W(cudaMalloc(&fr_src, sizeof(int) * kWide * (size_t)m));
-        DW_W(cudaMalloc(&n_inner, sizeof(int) * ((size_t)m + 1)));
-        DW_W(cudaMalloc(&offset, sizeof(int) * ((size_t)m + 1)));
-        wide_level_kernel<<<nblk(m, 128), 128, 0, s>>>(b.node_child, b.node_count, b.node_count + n_int,
-                                                       b.leaf_parent, roots, m, fr_code, fr_src, n_inner);
-        DW_W(cudaMemsetAsync(n_inner + m, 0, sizeof(int), s));
-        size_t tmp = 0;
-        DW_W(cub::DeviceScan::ExclusiveSum(nullptr, tmp, n_inner, offset, m + 1, s));
-        void* tmp_buf = nullptr;
-        DW_W(cudaMalloc(&tmp_buf, tmp));
-        e = cub::DeviceScan::ExclusiveSum(tmp_buf, tmp, n_inner, offset, m + 1, s);
-        int next_m = 0;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&next_m, offset + m, sizeof(int), cudaMemcpyDeviceToHost, s);
+    // level counts: one node (the binary root, id 0) at level 0
+    cudaError_t e = cudaMemsetAsync(b.wlev, 0, sizeof(int) * kWideLevels, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b.wroot, 0, sizeof(int), s);
+    int lev[kWideLevels] = {1};
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b.wlev, lev, sizeof(int), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    int done = 0;
+    while (done < kMax && lev[done] > 0) {        // a few levels at a time (200k triangles have eight, 4k segments three)
+        for (const int to = done + (DIM == 2 ? 4 : 9); done < to && done < kMax; ++done) {
+            long long most = 1;
+            for (int k = 0; k < done && most < n_int; ++k) most *= W;
+            const int blocks = min(nblk(most < n_int ? most : n_int, 128), 1024);
+            wide_level_kernel<W><<<blocks, 128, 0, s>>>(b.node_child, b.node_count, b.node_count + n_int,
+                                                        b.leaf_parent, done, b.wlev, b.wroot, b.wroot + n_int);
+        }
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(lev, b.wlev, sizeof(lev), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        cudaFree(tmp_buf);
-        if (e != cudaSuccess) { cleanup(); return e; }
-        cudaFree(next);
-        next = nullptr;
-        if (next_m > 0) DW_W(cudaMalloc(&next, sizeof(int) * (size_t)next_m));
-        wide_assign_kernel<<<nblk(m, 128), 128, 0, s>>>(fr_code, fr_src, offset, m, base + m, lc, ls, next);
-        DW_W(cudaGetLastError());
-        base += m;
-        m = next_m;
-        std::swap(roots, next);
+        if (e != cudaSuccess) return e;
     }
-    const int n_wide = base;
-    if (n_wide > b.wide_cap) {
+    b.n_wide = 0;
+    b.wide_depth = 0;
+    for (int l = 0; l < done && lev[l] > 0; ++l) { b.n_wide += lev[l]; b.wide_depth = l + 1; }
+    b.wide_ok = lev[kMax] == 0;
+    if (!b.wide_ok) { b.n_wide = 0; return cudaSuccess; }     // too deep: the binary tree serves every query
+    if (b.n_wide > b.wide_cap) {
         cudaFree(b.wnodes); cudaFree(b.wsrc);
         b.wnodes = nullptr; b.wsrc = nullptr; b.wide_cap = 0;
-        DW_W(cudaMalloc(&b.wnodes, sizeof(float) * WideLayout<3>::kFloats * (size_t)n_wide));
-        DW_W(cudaMalloc(&b.wsrc, sizeof(int) * 2 * kWide * (size_t)n_wide));   // sources, then codes
-        b.wide_cap = n_wide;
+        e = cudaMalloc(&b.wnodes, sizeof(float) * kNodeFloats * (size_t)b.n_wide);
+        if (e == cudaSuccess) e = cudaMalloc(&b.wsrc, sizeof(int) * (2 * W + 1) * (size_t)b.n_wide);
+        if (e != cudaSuccess) return e;
+        b.wide_cap = b.n_wide;
     }
-    b.n_wide = n_wide;
-    b.wide_depth = depth;
-    b.wide_ok = 31 * b.wide_depth + 1 <= kWideStack;
-    int* wcode = b.wsrc + kWide * (size_t)n_wide;
-    size_t at = 0;
-    for (size_t l = 0; l < lv_m.size(); ++l) {
-        const size_t n = kWide * (size_t)lv_m[l];
-        DW_W(cudaMemcpyAsync(b.wsrc + at, lv_src[l], sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
-        DW_W(cudaMemcpyAsync(wcode + at, lv_code[l], sizeof(int) * n, cudaMemcpyDeviceToDevice, s));
-        at += n;
-    }
-    wide_refit_kernel<DIM><<<nblk((long long)n_wide * kWide, 256), 256, 0, s>>>(b.nodes, b.prims, b.wsrc, wcode,
-                                                                               n_wide, b.wnodes);
-    DW_W(cudaGetLastError());
-    DW_W(cudaStreamSynchronize(s));      // the level buffers are freed next
-    cleanup();
-#undef DW_W
-    return cudaSuccess;
+    wide_codes_kernel<W><<<nblk(b.n_wide, 128), 128, 0, s>>>(
+        b.node_child, b.node_count, b.node_count + n_int, b.leaf_parent, b.n_wide, b.wroot, b.wroot + n_int,
+        b.wsrc + W * (size_t)b.n_wide, b.wsrc, b.wsrc + 2 * W * (size_t)b.n_wide);
+    return fill_wide<DIM>(b, s);
 }
 
 template <int DIM>
@@ -983,9 +1167,10 @@ static cudaError_t refit_impl(BvhBuffers& b, const float* vert, const int* elem,
         finalize_kernel<DIM><<<nblk(n, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, n, b.node_child,
                                                           b.node_parent, nt - 1, b.nodes, b.prims, b.prim_elem,
                                                           b.leaf_of_elem);
-        if (b.n_wide > 0)
-            wide_refit_kernel<DIM><<<nblk((long long)b.n_wide * kWide, 256), 256, 0, s>>>(
-                b.nodes, b.prims, b.wsrc, b.wsrc + kWide * (size_t)b.n_wide, b.n_wide, b.wnodes);
+        if (b.n_wide > 0) {
+            e = fill_wide<DIM>(b, s);
+            if (e != cudaSuccess) return e;
+        }
     } else {
         if (nt == 1) single_leaf_kernel<DIM><<<1, 1, 0, s>>>(vert, elem, b.vals_sorted, b.nodes, b.leaf_parent,
                                                              b.node_cell);
@@ -1021,9 +1206,10 @@ cudaError_t launch_closest(const BvhBuffers& b, int n, const float* p, const int
     BvhView v = view_of(b);
     if (traversal == 2 && b.wide_ok) {
         const WideView wv{b.wnodes, b.prims, b.n_wide, b.n_tree};
-        const size_t smem = sizeof(float2) * kWideStack * (128 / 32);
-        if (b.dim == 2) closest_wide_kernel<2><<<nblk(n, 128), 128, smem, s>>>(v, wv, b.prim_elem, b.leaf_of_elem, n, p, hint_elem, dist, elem_out, bary, err, ctr);
-        else closest_wide_kernel<3><<<nblk(n, 128), 128, smem, s>>>(v, wv, b.prim_elem, b.leaf_of_elem, n, p, hint_elem, dist, elem_out, bary, err, ctr);
+        const int cap = wide_stack_entries(b.dim, b.wide_depth);
+        const size_t smem = wide_smem_bytes(b.dim, cap) * (128 / 32);
+        if (b.dim == 2) closest_wide_kernel<2><<<nblk(n, 128), 128, smem, s>>>(v, wv, b.prim_elem, b.leaf_of_elem, n, p, hint_elem, dist, elem_out, bary, err, ctr, cap);
+        else closest_wide_kernel<3><<<nblk(n, 128), 128, smem, s>>>(v, wv, b.prim_elem, b.leaf_of_elem, n, p, hint_elem, dist, elem_out, bary, err, ctr, cap);
         return cudaGetLastError();
     }
     v.climb = traversal == 1 ? 1 : 0;

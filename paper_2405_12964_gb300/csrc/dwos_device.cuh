@@ -194,19 +194,28 @@ __device__ __forceinline__ float tri_closest(const float* q, const float3 a, con
     const float vc = fmaf(d1, d4, -__fmul_rn(d3, d2));
     const float vb = fmaf(d5, d2, -__fmul_rn(d1, d6));
     const float va = fmaf(d3, d6, -__fmul_rn(d5, d4));
-    float s, t;
-    if (d1 <= 0.0f && d2 <= 0.0f) { s = 0.0f; t = 0.0f; }                          // vertex a
-    else if (d3 >= 0.0f && d4 <= d3) { s = 1.0f; t = 0.0f; }                        // vertex b
-    else if (vc <= 0.0f && d1 >= 0.0f && d3 <= 0.0f) { s = __fdividef(d1, d1 - d3); t = 0.0f; }  // edge ab
-    else if (d6 >= 0.0f && d5 <= d6) { s = 0.0f; t = 1.0f; }                        // vertex c
-    else if (vb <= 0.0f && d2 >= 0.0f && d6 <= 0.0f) { s = 0.0f; t = __fdividef(d2, d2 - d6); }  // edge ac
-    else if (va <= 0.0f && (d4 - d3) >= 0.0f && (d5 - d6) >= 0.0f) {                // edge bc
-        const float u = __fdividef(d4 - d3, (d4 - d3) + (d5 - d6));
-        s = 1.0f - u; t = u;
-    } else {                                                                          // face
-        const float inv = __fdividef(1.0f, va + vb + vc);
-        s = __fmul_rn(vb, inv); t = __fmul_rn(vc, inv);
-    }
+    // The region's weights by selection, with one division whose operands depend on the
+    // region: the lanes of a warp lie in different regions, and as branches they ran one
+    // after the other with a division each.
+    const float g43 = d4 - d3, g56 = d5 - d6;
+    const bool in_a = d1 <= 0.0f && d2 <= 0.0f;
+    const bool in_b = d3 >= 0.0f && d4 <= d3;
+    const bool on_ab = vc <= 0.0f && d1 >= 0.0f && d3 <= 0.0f;
+    const bool in_c = d6 >= 0.0f && d5 <= d6;
+    const bool on_ac = vb <= 0.0f && d2 >= 0.0f && d6 <= 0.0f;
+    const bool on_bc = va <= 0.0f && g43 >= 0.0f && g56 >= 0.0f;
+    float num = 1.0f, den = va + vb + vc;                       // face
+    if (on_bc) { num = g43; den = g43 + g56; }
+    if (on_ac) { num = d2; den = d2 - d6; }
+    if (on_ab) { num = d1; den = d1 - d3; }
+    const float r = __fdividef(num, den);
+    float s = __fmul_rn(vb, r), t = __fmul_rn(vc, r);           // face
+    if (on_bc) { s = 1.0f - r; t = r; }                         // edge bc
+    if (on_ac) { s = 0.0f; t = r; }                             // edge ac
+    if (in_c) { s = 0.0f; t = 1.0f; }                           // vertex c
+    if (on_ab) { s = r; t = 0.0f; }                             // edge ab
+    if (in_b) { s = 1.0f; t = 0.0f; }                           // vertex b
+    if (in_a) { s = 0.0f; t = 0.0f; }                           // vertex a
     const float rx = fmaf(-t, ac.x, fmaf(-s, ab.x, ap.x));
     const float ry = fmaf(-t, ac.y, fmaf(-s, ab.y, ap.y));
     const float rz = fmaf(-t, ac.z, fmaf(-s, ab.z, ap.z));
@@ -460,7 +469,7 @@ __device__ __forceinline__ float gradient_factor(float k, float R) {
     return 2.0f * k * z * z * expf(-z) / (z - 1.0f);   // i1(z) = e^z (z - 1) / (2 z^2) + O(e^-z)
 }
 
-// ---- 32-wide BVH searched by a whole warp ---------------------------------
+// ---- 32-wide BVH of segments, searched by a whole warp ----------------------
 // The binary LBVH collapsed five levels at a time: a wide node holds up to 32
 // children in SoA order, lo[DIM][32], hi[DIM][32], code[32] (>= 0: wide node,
 // < 0: ~leaf, kEmptyChild: unused slot with an empty box) and, for leaf
@@ -477,7 +486,7 @@ template <int DIM> struct WideLayout {
 };
 
 struct WideView {
-    const float* wnodes;   // n_wide nodes of WideLayout<DIM>::kFloats floats, root first
+    const float* wnodes;   // n_wide nodes, root first (2D: WideLayout, 3D: oriented nodes)
     const float4* prims;
     int n_wide;
     int n_tree;
@@ -591,6 +600,276 @@ __device__ __forceinline__ int wide_closest(const WideView& mine, unsigned need,
         if (lane == src) { best2 = b2; best = bi; }
     }
     return err;
+}
+
+// ---- 8-wide BVH of triangles with oriented boxes, searched by groups of lanes ---
+// The binary LBVH collapsed three levels at a time.  A node is eight child slots, one
+// per lane of a group of eight lanes; slot j is an oriented box (centre c, orthonormal
+// rows r, half extents h) with the child's code (>= 0: node, < 0: ~leaf, kEmptyChild:
+// unused), [c.xyz code] [r0.xyz h.0] [r1.xyz h.1] [r2.xyz h.2], its float4 k at
+// k * 8 + j, so that a group reads consecutive addresses.
+// A patch of a finely cut surface is thin along its own normal but fills its
+// axis-aligned box, and a distant query then finds the boxes of many patches closer
+// than its closest element: over a 200k-triangle sphere 20.7 visits per query of a
+// 32-wide tree with axis-aligned boxes against 8.2 with oriented ones, of an 8-wide
+// one 48 against 15.  Width and grouping by measurement (walk kernel of 4.2 M walks over
+// that sphere / of 3,200 walks over 5,800 triangles, ms): one query at a time on 32
+// axis-aligned slots 91.5 / 0.45, on 32 oriented ones 63 / 0.44, two at a time on 16 57 /
+// 0.50, four on 8 48.8 / 0.60 (kept), eight on 4 49.0 / 0.70.
+constexpr int kOriented = 8;               // slots of a node, lanes of a group
+constexpr int kOrientedF4 = 4 * kOriented;
+constexpr int kOrientedDepthMax = 12;      // levels (checked at build)
+// Leaves measured together, at least (16 / 24 / 32: 48.8 / 49.6 / 51.9 ms).
+constexpr int kCandFlush = 16;
+
+// A warp's shared memory for the search, followed by a stack of stk_cap entries
+// (distance and code) for each group: per lane the closest element so far (its squared
+// distance's bits and its leaf), and the leaves that wait to be measured with the lane
+// whose query they belong to.
+struct SearchScratch {
+    unsigned dist[32], leaf[32];
+    unsigned cand[kCandFlush + 32];
+    unsigned char cand_lane[kCandFlush + 32];
+};
+static_assert(sizeof(SearchScratch) % 8 == 0, "the stacks follow");
+// Stack entries of one group: each level leaves at most seven siblings behind.
+__host__ __device__ inline int oriented_stack_entries(int depth) { return (kOriented - 1) * depth + 1; }
+__host__ __device__ inline size_t oriented_smem_bytes(int stk_cap) {   // per warp
+    return sizeof(SearchScratch) + sizeof(float2) * (32 / kOriented) * (size_t)stk_cap;
+}
+
+// Squared distance from q to an oriented box.  q - c is rounded relative to the
+// distance itself, and the half extents carry a margin for the rest (build), so
+// that the result exceeds the true distance by less than `within` allows.
+__device__ __forceinline__ float obb_dist2(const float* q, const float4* s) {
+    const float dx = q[0] - s[0].x, dy = q[1] - s[0].y, dz = q[2] - s[0].z;
+    float d = 0.0f;
+#pragma unroll
+    for (int k = 1; k < 4; ++k) {
+        const float e = fmaxf(fabsf(fmaf(s[k].x, dx, fmaf(s[k].y, dy, s[k].z * dz))) - s[k].w, 0.0f);
+        d = fmaf(e, e, d);
+    }
+    return d;
+}
+
+// Closest tree leaf for every lane in `need`: four queries at a time, each on a
+// group of eight lanes.  A group that runs out of nodes takes the next waiting query,
+// or, when none waits, a node from another group's stack (the ends of the longest
+// searches of a warp step are shared: 53.3 -> 50.2 ms).  Lane j of a group tests child
+// slot j of the group's current node; the
+// nearest inner child that can still hold a closer leaf is visited next, the
+// others go on the group's stack in shared memory, and a pop looks at the top
+// eight entries at once for the first that is still within the bound.  Leaf
+// children within the bound go on the warp's list and are measured one per lane
+// when kCandFlush or more wait, whichever queries they belong to: an element's
+// distance costs more instructions than a visit, and at each visit only a few
+// lanes of the warp hold a leaf (63.3 -> 53.3 ms).  Each lane's closest element so far
+// lives in shared
+// memory (two 32-bit minima: the distance's bits, then the lower leaf index among
+// equals, the order of `closer`), so that groups need not wait for their leaves and
+// several can serve one query.
+// n_nodes counts node visits, n_prims measured leaves.
+// best2 / best hold each lane's bound on entry (kInf / -1 without one) and
+// the result on exit.  Called by all 32 lanes with the same `need` and each
+// lane's own view (lanes may belong to different problems).  Returns 1 if a
+// group visited more nodes than a query's budget or would overflow its stack
+// (excluded by the stack's size for the tree's depth), which ends its search.
+__device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned need, const float* q_lane, float& best2,
+                                                int& best, SearchScratch* sc, int stk_cap, unsigned& n_nodes,
+                                                unsigned& n_prims) {
+    const int lane = threadIdx.x & 31;
+    constexpr int DIM = 3, W = kOriented;
+    constexpr unsigned kGroupBits = (1u << W) - 1u, kHeads = 0x01010101u;   // the groups' first lanes
+    const int gb = lane & ~(W - 1), j = lane & (W - 1);
+    const unsigned below = (1u << lane) - 1u;
+    float2* st = reinterpret_cast<float2*>(sc + 1) + (gb / W) * stk_cap;
+    int err = 0;
+    // one-leaf trees have no wide nodes: each lane measures its own
+    const unsigned lone = __ballot_sync(kWarpAll, mine.n_wide == 0);
+    if (((need >> lane) & 1u) && mine.n_wide == 0 && mine.n_tree == 1) {
+        const float dd = prim_dist2<DIM>(mine.prims, 0, q_lane);
+        ++n_prims;
+        if (closer(dd, 0, best2, best)) { best2 = dd; best = 0; }
+    }
+    unsigned rest = need & ~lone;      // queries that wait (the same in every lane)
+    if (rest == 0) return 0;
+    sc->dist[lane] = __float_as_uint(best2);
+    sc->leaf[lane] = (unsigned)best;
+    float q[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) q[k] = 0.0f;
+    int src = 0, top = 0, cur = -1, budget = 0, n_cand = 0;
+    const float4* wn = reinterpret_cast<const float4*>(mine.wnodes);
+    __syncwarp();
+    // measures the listed leaves, one per lane
+    auto flush = [&]() {
+        while (n_cand > 0) {
+            n_cand -= 32;
+            const int at = n_cand + lane;
+            const bool has = at >= 0;
+            const int s = has ? sc->cand_lane[at] : 0;
+            const unsigned p = has ? sc->cand[at] : 0u;
+            float qs[DIM];
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) qs[k] = __shfl_sync(kWarpAll, q_lane[k], s);
+            const float4* prims = reinterpret_cast<const float4*>(
+                __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.prims), s));
+            unsigned bits = 0xffffffffu;
+            if (has) {
+                ++n_prims;
+                const float dd = prim_dist2<DIM>(prims, (int)p, qs);
+                if (dd < kInf) bits = __float_as_uint(dd);    // squared distances are >= 0: bits order like values
+            }
+            const unsigned old = sc->dist[s];
+            __syncwarp();
+            if (bits < old) atomicMin(&sc->dist[s], bits);
+            __syncwarp();
+            const unsigned now = sc->dist[s];
+            if (bits == now && now < old) sc->leaf[s] = 0xffffffffu;
+            __syncwarp();
+            if (bits == now) atomicMin(&sc->leaf[s], p);
+            __syncwarp();
+        }
+        n_cand = 0;
+    };
+    for (;;) {
+        const unsigned idle = __ballot_sync(kWarpAll, cur < 0 && top == 0);
+        if (idle) {
+            if (rest) {   // the k-th idle group takes the k-th waiting query
+                unsigned heads = idle & kHeads, m = rest;
+                for (int k = __popc(heads & ((1u << gb) - 1u)); k > 0; --k) m &= m - 1u;
+                const bool take = ((idle >> lane) & 1u) && m;
+                const int s = m ? __ffs(m) - 1 : 0;
+                for (; heads && rest; heads &= heads - 1u) rest &= rest - 1u;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    const float v = __shfl_sync(kWarpAll, q_lane[k], s);
+                    if (take) q[k] = v;
+                }
+                const unsigned long long vp = __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.wnodes), s);
+                const int vb = __shfl_sync(kWarpAll, mine.budget > 0 ? mine.budget : mine.n_wide, s);
+                if (take) {
+                    src = s;
+                    wn = reinterpret_cast<const float4*>(vp);
+                    budget = vb;
+                    cur = 0;
+                }
+            } else if (idle == kWarpAll) {
+                break;
+            } else {
+                // no query waits: the k-th idle group takes the top entry of the k-th busy group
+                // that has one, and goes on with that group's query
+                const unsigned heads = idle & kHeads;
+                const unsigned busy = __ballot_sync(kWarpAll, top > 0) & kHeads;
+                const unsigned under = (1u << gb) - 1u;
+                if (busy) {
+                    const int rank = __popc(heads & under);
+                    unsigned m = busy;
+                    for (int k = rank; k > 0; --k) m &= m - 1u;
+                    const bool take = ((idle >> lane) & 1u) && m;
+                    const int v = take ? __ffs(m) - 1 : gb;
+                    const int vtop = __shfl_sync(kWarpAll, top, v);
+                    const float2 e = st[(v - gb) / W * stk_cap + (vtop > 0 ? vtop - 1 : 0)];
+                    const int vsrc = __shfl_sync(kWarpAll, src, v), vbud = __shfl_sync(kWarpAll, budget, v);
+                    const unsigned long long vp = __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(wn), v);
+#pragma unroll
+                    for (int k = 0; k < DIM; ++k) {
+                        const float t = __shfl_sync(kWarpAll, q[k], v);
+                        if (take) q[k] = t;
+                    }
+                    if (((busy >> gb) & 1u) && __popc(busy & under) < __popc(heads)) --top;
+                    if (take) {
+                        src = vsrc;
+                        budget = vbud;
+                        wn = reinterpret_cast<const float4*>(vp);
+                        cur = within(e.x, __uint_as_float(sc->dist[vsrc])) ? __float_as_int(e.y) : -1;
+                    }
+                }
+            }
+        }
+        const float b2 = __uint_as_float(sc->dist[src]);
+        {   // pop: the topmost of the top four entries that is still within the bound
+            const int at = top - 1 - j;
+            const bool look = cur < 0 && at >= 0;
+            const float2 e = look ? st[at] : make_float2(kInf, 0.0f);
+            const unsigned ok = (__ballot_sync(kWarpAll, look && within(e.x, b2)) >> gb) & kGroupBits;
+            const int first = ok ? __ffs(ok) - 1 : 0;
+            const int code = __shfl_sync(kWarpAll, __float_as_int(e.y), gb + first);
+            if (cur < 0) {
+                cur = ok ? code : -1;
+                top = ok ? top - 1 - first : max(top - W, 0);
+            }
+        }
+        // visit
+        const bool go = cur >= 0;
+        int code = kEmptyChild;
+        float cd = kInf;
+        if (go) {
+            if (j == 0) ++n_nodes;
+            const float4* f = wn + (size_t)cur * kOrientedF4 + j;
+            float4 s[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) s[k] = __ldg(f + k * W);
+            code = __float_as_int(s[0].w);
+            cd = obb_dist2(q, s);
+            if (--budget < 0) { err = 1; code = kEmptyChild; top = 0; }
+        }
+        const bool ok = code != kEmptyChild && within(cd, b2);
+        const bool inner = ok && code >= 0;
+        const unsigned lm = __ballot_sync(kWarpAll, ok && code < 0);
+        const unsigned im = (__ballot_sync(kWarpAll, inner) >> gb) & kGroupBits;
+        if (lm) {
+            if ((lm >> lane) & 1u) {
+                const int at = n_cand + __popc(lm & below);
+                sc->cand[at] = (unsigned)~code;
+                sc->cand_lane[at] = (unsigned char)src;
+            }
+            n_cand += __popc(lm);
+        }
+        // the nearest inner child (the low bits of its distance give way to its slot)
+        unsigned key = inner ? (__float_as_uint(cd) & ~(unsigned)(W - 1)) | (unsigned)j : 0xffffffffu;
+#pragma unroll
+        for (int o = 1; o < W; o <<= 1) key = min(key, __shfl_xor_sync(kWarpAll, key, o));
+        const int ml = (int)(key & (W - 1));
+        const int next = __shfl_sync(kWarpAll, code, gb + ml);
+        const unsigned others = im & ~(1u << ml);
+        if (go) {
+            cur = im ? next : -1;
+            if (top + __popc(others) > stk_cap) { err = 1; cur = -1; top = 0; }
+            else {
+                if (inner && j != ml)
+                    st[top + __popc(others & ((1u << j) - 1u))] = make_float2(cd, __int_as_float(code));
+                top += __popc(others);
+            }
+        }
+        __syncwarp();
+        if (n_cand >= kCandFlush) flush();
+    }
+    flush();
+    best2 = __uint_as_float(sc->dist[lane]);
+    best = (int)sc->leaf[lane];
+    __syncwarp();
+    return err;
+}
+
+// A warp's search of the wide tree and its shared memory (stk_cap: from
+// wide_stack_entries; the 2D stack's size is fixed).
+__host__ __device__ inline int wide_stack_entries(int dim, int depth) {
+    return dim == 2 ? kWideStack : oriented_stack_entries(depth > 0 ? depth : 1);
+}
+__host__ __device__ inline size_t wide_smem_bytes(int dim, int stk_cap) {   // per warp
+    return dim == 2 ? sizeof(float2) * kWideStack : oriented_smem_bytes(stk_cap);
+}
+template <int DIM>
+__device__ __forceinline__ int wide_search(const WideView& mine, unsigned need, const float* q, float& best2, int& best,
+                                           float2* stk, int stk_cap, unsigned& n_nodes, unsigned& n_prims) {
+    if constexpr (DIM == 2) return wide_closest<DIM>(mine, need, q, best2, best, stk, n_nodes, n_prims);
+    else return oriented_closest(mine, need, q, best2, best, reinterpret_cast<SearchScratch*>(stk), stk_cap, n_nodes, n_prims);
+}
+
+// Wide nodes in units of 32 child slots, as the statistics report them.
+__host__ __device__ inline unsigned long long wide_units(int dim, unsigned long long n) {
+    return dim == 2 ? n : (n * kOriented + 31) / 32;
 }
 
 // Outsized elements (kept out of the tree) against one lane's query.

@@ -64,10 +64,10 @@ struct DevProblem {
     const int* leaf_parent;     // leaf -> parent node
     const float* node_cell;     // Morton cell per internal node
     float r_max;                // element radius bound for the cell test
-    int traversal;              // 0 root-down, 1 climb from the hint leaf, 2 warp-wide over the 32-wide tree,
+    int traversal;              // 0 root-down, 1 climb from the hint leaf, 2 by the warp over the wide tree,
                                 // 3 routed: no tree search if the binary root's child boxes are outside the
-                                // bound, else warp-wide (per lane when many lanes need one in a step)
-    const float* wnodes;        // 32-wide tree (SoA nodes), root first
+                                // bound, else as 2 (2D: per lane for small trees and when many lanes need one)
+    const float* wnodes;        // wide tree (2D 32-wide, 3D 8-wide nodes), root first
     int n_wide;                 // its node count
     int data_kind;              // 0 mapped, 1 field
     int differential;
@@ -116,7 +116,7 @@ struct DevCounters {
     unsigned long long capped;
     unsigned long long nodes;   // binary BVH node fetches
     unsigned long long prims;   // element distance tests
-    unsigned long long wnodes;  // 32-wide node visits
+    unsigned long long wnodes;  // wide node visits
     int error;                  // bit 0: traversal bound exceeded, bit 1: query outside Omega,
                                 // bit 2: query point not finite
     int pad[1];
@@ -149,9 +149,13 @@ struct BvhBuffers {
     void* sort_tmp = nullptr;
     size_t sort_tmp_bytes = 0;
     int capacity = 0;
-    // 32-wide tree collapsed from the binary one (rebuilt with it), nodes in level order
-    float* wnodes = nullptr;         // n_wide x WideLayout<dim>::kFloats
-    int* wsrc = nullptr;             // per slot: (binary parent << 1 | side) of the child's box, -1 unused
+    // wide tree collapsed from the binary one (rebuilt with it), nodes level by level
+    float* wnodes = nullptr;         // n_wide nodes (2D WideLayout, 3D kOrientedF4 float4)
+    int* wsrc = nullptr;             // per slot: (binary parent << 1 | side) of the child's box, -1 unused; then per
+                                     // slot its code; then per node the slot that holds it
+    int* wroot = nullptr;            // per wide node: the binary node it was collapsed from; then the id of its
+                                     // first inner child
+    int* wlev = nullptr;             // wide nodes per level
     int n_wide = 0, wide_depth = 0, wide_cap = 0;
     bool wide_ok = false;            // the warp-wide search fits its stack on this tree
 };
@@ -161,7 +165,7 @@ void bvh_free(BvhBuffers& b);
 cudaError_t bvh_build(BvhBuffers& b, int dim, const float* vert, const int* elem, int n_elem,
                       cudaStream_t stream);
 // New boxes for moved vertices over the same elements and tree topology (binary
-// and 32-wide): every box again bounds its subtree, so the exact searches of
+// and wide): every box again bounds its subtree, so the exact searches of
 // orders 0, 2 and 3 stay exact; no host synchronisation and no allocation.
 // The Morton cells go stale (cells_ok = false).
 cudaError_t bvh_refit(BvhBuffers& b, const float* vert, const int* elem, cudaStream_t stream);
@@ -186,7 +190,8 @@ struct WalkLaunch {
     int block_size;
     int blocks_per_sm;
     int n_sm;
-    int traversal = 0;          // 2, 3: warp-wide search (every problem of the launch has wide_ok)
+    int traversal = 0;          // 2, 3: search by the warp (every problem of the launch has wide_ok)
+    int wide_depth = 0;         // levels of the deepest wide tree among them
     bool star = false;          // walk on stars (one problem with a Neumann part)
     bool cones = false;         // walk on stars whose silhouette tree has normal cones
     bool data = false;          // walk on stars with Neumann data (runs without the cones)
@@ -198,8 +203,7 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
                          unsigned long long total_work, DevCounters* d_counters, cudaStream_t stream,
                          int* blocks_used, const DevProblem* host_prob = nullptr,
                          DevCounters* zero_counters = nullptr);
-int walk_max_blocks_per_sm(int dim, int block_size, int traversal = 0, bool star = false, bool cones = false,
-                           bool data = false);
+int walk_max_blocks_per_sm(const WalkLaunch& L);
 // Query points on the Neumann part: per point the closest Neumann element if it
 // lies within tol of it (q_start w = its compact index, xyz = its unit normal,
 // not yet oriented) and the point 1e-3 of the element's size behind its centre

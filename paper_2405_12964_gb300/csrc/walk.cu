@@ -94,14 +94,14 @@ struct PhaseState {
     uint32_t pad[DIM == 2 ? 1 : 2];      // 19 / 23 words
 };
 
-// Dynamic shared memory: the problem descriptors, then (warp-wide search only)
-// one traversal stack per warp and the threads' phase states, or (walk on
+// Dynamic shared memory: the problem descriptors, then (search by the warp only: stk_cap
+// > 0) the warps' search areas and the threads' phase states, then (walk on
 // stars) the Neumann part's descriptor.
-__host__ __device__ inline size_t walk_smem_bytes(int n_probs, int block_size, int traversal, int dim = 3,
+__host__ __device__ inline size_t walk_smem_bytes(int n_probs, int block_size, int stk_cap, int dim = 3,
                                                   bool star = false) {
     size_t b = (sizeof(DevProblem) * (size_t)n_probs + 15) & ~(size_t)15;
-    if (traversal == 2 || traversal == 3)
-        b += sizeof(float2) * kWideStack * (size_t)(block_size / 32) +
+    if (stk_cap > 0)
+        b += wide_smem_bytes(dim, stk_cap) * (size_t)(block_size / 32) +
              (dim == 2 ? sizeof(PhaseState<2>) : sizeof(PhaseState<3>)) * (size_t)block_size;
     if (star) b += sizeof(DevNeumann);
     return b;
@@ -131,15 +131,16 @@ __device__ __forceinline__ void sphere_dir(const U4& r, float* om) {
 template <int DIM, bool WIDE, bool STAR = false, bool CONES = false, bool DATA = false>
 __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
     walk_kernel(const DevProblem* __restrict__ g_probs, int n_probs, unsigned long long total,
-                DevCounters* __restrict__ ctr, DevCounters* __restrict__ zero_ctr, int lanes,
-                const __grid_constant__ DevProblem p_arg) {
+                DevCounters* __restrict__ ctr, DevCounters* __restrict__ zero_ctr, int stk_cap,
+                int lanes, const __grid_constant__ DevProblem p_arg) {
     constexpr bool wide = WIDE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     DevProblem* sp = reinterpret_cast<DevProblem*>(smem_raw);
     float2* stk_base = reinterpret_cast<float2*>(smem_raw + walk_smem_bytes(n_probs, 0, 0));
-    float2* stk = stk_base + (size_t)(threadIdx.x >> 5) * kWideStack;
+    const int warp_area = (int)(wide_smem_bytes(DIM, stk_cap) / sizeof(float2));
+    float2* stk = stk_base + (size_t)(threadIdx.x >> 5) * warp_area;
     PhaseState<DIM> ps_reg;
-    PhaseState<DIM>& S = WIDE ? reinterpret_cast<PhaseState<DIM>*>(stk_base + (size_t)(blockDim.x >> 5) * kWideStack)[threadIdx.x]
+    PhaseState<DIM>& S = WIDE ? reinterpret_cast<PhaseState<DIM>*>(stk_base + (size_t)(blockDim.x >> 5) * warp_area)[threadIdx.x]
                               : ps_reg;
     {
         // the descriptor table, or the one problem passed by value
@@ -154,8 +155,8 @@ __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
     }
     __syncthreads();
     // the Neumann descriptor follows the problems (and, warp-wide, the stacks and phase states)
-    DevNeumann& NS = *reinterpret_cast<DevNeumann*>(smem_raw + walk_smem_bytes(n_probs, WIDE ? (int)blockDim.x : 0,
-                                                                               WIDE ? 3 : 0, DIM, false));
+    DevNeumann& NS = *reinterpret_cast<DevNeumann*>(smem_raw + walk_smem_bytes(n_probs, (int)blockDim.x, WIDE ? stk_cap : 0,
+                                                                               DIM, false));
     if constexpr (STAR) {
         const int words = (int)(sizeof(DevNeumann) / sizeof(int));
         const int* src = reinterpret_cast<const int*>(sp[0].neu);
@@ -270,9 +271,9 @@ __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
                     need = __ballot_sync(kFull, desc && !lane_search);
                 }
             }
-            if (need) {   // all lanes search the 32-wide tree together, one lane's query at a time
+            if (need) {   // the lanes search the wide tree together
                 const WideView wv{Pw.wnodes, Pw.prims, Pw.n_wide, Pw.n_tree, Pw.node_budget};
-                error |= wide_closest<DIM>(wv, need, x, best2, best, stk, st.wnodes, st.prims) & 1;
+                error |= wide_search<DIM>(wv, need, x, best2, best, stk, stk_cap, st.wnodes, st.prims) & 1;
             }
         }
         if (!active) continue;
@@ -791,29 +792,44 @@ cudaError_t launch_neumann_orient(int n, const int* behind_inside, float4* q_sta
     return cudaGetLastError();
 }
 
-int walk_max_blocks_per_sm(int dim, int block_size, int traversal, bool star, bool cones, bool data) {
-    int n = 0;
-    const size_t smem = walk_smem_bytes(1, block_size, traversal, dim, star);
-    const bool wide = traversal == 2 || traversal == 3;
-    auto occ = [&](auto kernel) { cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, block_size, smem); };
-    if (star && data) {
-        if (dim == 2) wide ? occ(walk_kernel<2, true, true, false, true>) : occ(walk_kernel<2, false, true, false, true>);
-        else wide ? occ(walk_kernel<3, true, true, false, true>) : occ(walk_kernel<3, false, true, false, true>);
-    } else if (star) {
-        if (dim == 2) {
-            if (wide) cones ? occ(walk_kernel<2, true, true, true>) : occ(walk_kernel<2, true, true>);
-            else cones ? occ(walk_kernel<2, false, true, true>) : occ(walk_kernel<2, false, true>);
-        } else {
-            if (wide) cones ? occ(walk_kernel<3, true, true, true>) : occ(walk_kernel<3, true, true>);
-            else cones ? occ(walk_kernel<3, false, true, true>) : occ(walk_kernel<3, false, true>);
+namespace {
+
+bool wide_launch(const WalkLaunch& L) { return L.traversal == 2 || L.traversal == 3; }
+
+int stack_entries(const WalkLaunch& L) { return wide_launch(L) ? wide_stack_entries(L.dim, L.wide_depth) : 0; }
+
+// Calls f with the kernel instantiation of a launch.
+template <class F>
+cudaError_t with_kernel(const WalkLaunch& L, F f) {
+    const bool wide = wide_launch(L);
+    if (L.star) {
+        if (L.data) {   // normal cones only prune; the data instantiation runs without them
+            if (wide) return L.dim == 2 ? f(walk_kernel<2, true, true, false, true>) : f(walk_kernel<3, true, true, false, true>);
+            return L.dim == 2 ? f(walk_kernel<2, false, true, false, true>) : f(walk_kernel<3, false, true, false, true>);
         }
-    } else if (traversal == 2 || traversal == 3) {
-        if (dim == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<2, true>, block_size, smem);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<3, true>, block_size, smem);
-    } else {
-        if (dim == 2) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<2, false>, block_size, smem);
-        else cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, walk_kernel<3, false>, block_size, smem);
+        if (L.cones) {
+            if (wide) return L.dim == 2 ? f(walk_kernel<2, true, true, true>) : f(walk_kernel<3, true, true, true>);
+            return L.dim == 2 ? f(walk_kernel<2, false, true, true>) : f(walk_kernel<3, false, true, true>);
+        }
+        if (wide) return L.dim == 2 ? f(walk_kernel<2, true, true>) : f(walk_kernel<3, true, true>);
+        return L.dim == 2 ? f(walk_kernel<2, false, true>) : f(walk_kernel<3, false, true>);
     }
+    if (wide) return L.dim == 2 ? f(walk_kernel<2, true>) : f(walk_kernel<3, true>);
+    return L.dim == 2 ? f(walk_kernel<2, false>) : f(walk_kernel<3, false>);
+}
+
+}  // namespace
+
+int walk_max_blocks_per_sm(const WalkLaunch& L) {
+    int n = 0;
+    const size_t smem = walk_smem_bytes(1, L.block_size, stack_entries(L), L.dim, L.star);
+    with_kernel(L, [&](auto kernel) {
+        if (smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, L.block_size, smem);
+    });
     return n;
 }
 
@@ -830,8 +846,7 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
     const int bs = L.block_size;
     if (bs % 32 != 0) return cudaErrorInvalidValue;
     if (L.star && n_probs != 1) return cudaErrorInvalidValue;
-    int per_sm = L.blocks_per_sm > 0 ? L.blocks_per_sm
-                                     : walk_max_blocks_per_sm(L.dim, bs, L.traversal, L.star, L.cones, L.data);
+    int per_sm = L.blocks_per_sm > 0 ? L.blocks_per_sm : walk_max_blocks_per_sm(L);
     if (per_sm < 1) per_sm = 1;
     // A launch that cannot fill every lane spreads its walks over all warps, a few lanes
     // each: a warp's iteration lasts as long as its lanes' searches take in turn, and the
@@ -846,34 +861,19 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
     if (blocks > need) blocks = need;
     if (blocks < 1) blocks = 1;
     if (blocks_used) *blocks_used = (int)blocks;
-    const size_t smem = walk_smem_bytes(n_probs, bs, L.traversal, L.dim, L.star);
+    const int cap = stack_entries(L);
+    const size_t smem = walk_smem_bytes(n_probs, bs, cap, L.dim, L.star);
     DevProblem P1;
     if (host_prob) P1 = *host_prob;
     else memset(&P1, 0, sizeof(P1));
-    auto go = [&](auto kernel) -> cudaError_t {
+    return with_kernel(L, [&](auto kernel) -> cudaError_t {
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kernel<<<(int)blocks, bs, smem, stream>>>(d_probs, n_probs, total, d_counters, zero_counters, lanes, P1);
+        kernel<<<(int)blocks, bs, smem, stream>>>(d_probs, n_probs, total, d_counters, zero_counters, cap, lanes, P1);
         return cudaGetLastError();
-    };
-    if (L.star) {
-        const bool wide = L.traversal == 2 || L.traversal == 3;
-        if (L.data) {   // normal cones only prune; the data instantiation runs without them
-            if (wide) return L.dim == 2 ? go(walk_kernel<2, true, true, false, true>)
-                                        : go(walk_kernel<3, true, true, false, true>);
-            return L.dim == 2 ? go(walk_kernel<2, false, true, false, true>) : go(walk_kernel<3, false, true, false, true>);
-        }
-        if (L.cones) {
-            if (wide) return L.dim == 2 ? go(walk_kernel<2, true, true, true>) : go(walk_kernel<3, true, true, true>);
-            return L.dim == 2 ? go(walk_kernel<2, false, true, true>) : go(walk_kernel<3, false, true, true>);
-        }
-        if (wide) return L.dim == 2 ? go(walk_kernel<2, true, true>) : go(walk_kernel<3, true, true>);
-        return L.dim == 2 ? go(walk_kernel<2, false, true>) : go(walk_kernel<3, false, true>);
-    }
-    if (L.traversal == 2 || L.traversal == 3) return L.dim == 2 ? go(walk_kernel<2, true>) : go(walk_kernel<3, true>);
-    return L.dim == 2 ? go(walk_kernel<2, false>) : go(walk_kernel<3, false>);
+    });
 }
 
 }  // namespace dwos
