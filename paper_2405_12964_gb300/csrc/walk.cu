@@ -29,12 +29,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // Search order 3 routes each query by the binary root's two child boxes: most
 // queries (closer to an outsized element, or to their seed, than to any tree
 // box) need no tree search at all; the few that do are searched by the whole
-// warp over the 32-wide tree, one at a time.  Segments are searched one query per
-// lane, over the binary tree, where more than kLaneSearchMin lanes of the warp need
-// a search in the same step (16 or 33: within 2 % on a 4096-segment star whose
-// points' queries mostly need one) or the tree has at most kLaneTreeMax leaves (128
-// segments: 0.34 ms against 0.42 ms by groups of lanes); triangles never.
-constexpr int kLaneSearchMin = 16;
+// warp over the wide tree.  Trees of at most kLaneTreeMax segments are searched one
+// query per lane, over the binary tree (128 segments: 0.34 ms against 0.42 ms by groups
+// of lanes); for larger ones, and for triangles, that never pays (2.1 M walks around a
+// 4096-segment star, half of whose queries need the tree: 7.5 ms when steps with more
+// than 16 such lanes went one per lane, 6.4 ms without).
 constexpr int kLaneTreeMax = 256;
 
 template <int DIM>
@@ -267,7 +266,7 @@ __global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
                 }
                 need = __ballot_sync(kFull, desc);
                 if (DIM == 2) {
-                    lane_search = desc && (Pw.n_tree <= kLaneTreeMax || __popc(need) > kLaneSearchMin);
+                    lane_search = desc && Pw.n_tree <= kLaneTreeMax;
                     need = __ballot_sync(kFull, desc && !lane_search);
                 }
             }
