@@ -433,48 +433,19 @@ __global__ void wide_codes_kernel(const int* node_child, const int* node_count, 
     }
 }
 
-// Child boxes gathered from the binary tree (its refit already ran) and codes.
-template <int DIM>
+// The 2D tree's slots: inner children's boxes gathered from the binary tree (its refit
+// already ran), leaf children's segments, and the codes.
 __global__ void wide_refit_kernel(const float4* nodes, const float4* prims, const int* wsrc, const int* wcode,
                                   int n_wide, float* wnodes) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n_wide * kWide) return;
-    const int w = t / kWide, j = t % kWide;
-    float* f = wnodes + (size_t)w * WideLayout<DIM>::kFloats;
-    const int src = wsrc[t];
-    float lo[DIM], hi[DIM];
-    if (src < 0) {
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) { lo[k] = kInf; hi[k] = -kInf; }
-    } else {
-        const float* b = reinterpret_cast<const float*>(nodes + BvhLayout<DIM>::kNodeF4 * (src >> 1)) +
-                         (DIM == 2 ? 4 : 6) * (src & 1);
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) { lo[k] = b[k]; hi[k] = b[DIM + k]; }
-    }
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) { f[k * kWide + j] = lo[k]; f[(DIM + k) * kWide + j] = hi[k]; }
-    const int code = wcode[t];
-    f[2 * DIM * kWide + j] = __int_as_float(code);
-    // a leaf child's vertices (the element in Morton order), zeros otherwise
-    float v[DIM * DIM];
-#pragma unroll
-    for (int k = 0; k < DIM * DIM; ++k) v[k] = 0.0f;
-    if (code < 0) {
-        const int p = ~code;
-        if constexpr (DIM == 2) {
-            const float4 sgm = prims[p];
-            v[0] = sgm.x; v[1] = sgm.y; v[2] = sgm.z; v[3] = sgm.w;
-        } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float4 a = prims[3 * p + c];
-                v[3 * c] = a.x; v[3 * c + 1] = a.y; v[3 * c + 2] = a.z;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < DIM * DIM; ++k) f[WideLayout<DIM>::kVtx + k * kWide + j] = v[k];
+    float* f = wnodes + (size_t)(t / kWide) * kWideFloats;
+    const int j = t % kWide, src = wsrc[t], code = wcode[t];
+    float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (code < 0) v = prims[~code];
+    else if (src >= 0) v = nodes[BvhLayout<2>::kNodeF4 * (src >> 1) + (src & 1)];
+    reinterpret_cast<float4*>(f)[j] = v;
+    f[4 * kWide + j] = __int_as_float(code);
 }
 
 __device__ __forceinline__ float warp_fsum(float v) {
@@ -1026,7 +997,7 @@ constexpr int kMaxBig = 64;
 template <int DIM>
 static cudaError_t fill_wide(BvhBuffers& b, cudaStream_t s) {
     if constexpr (DIM == 2) {
-        wide_refit_kernel<DIM><<<nblk((long long)b.n_wide * kWide, 256), 256, 0, s>>>(
+        wide_refit_kernel<<<nblk((long long)b.n_wide * kWide, 256), 256, 0, s>>>(
             b.nodes, b.prims, b.wsrc, b.wsrc + kWide * (size_t)b.n_wide, b.n_wide, b.wnodes);
     } else {
         oriented_fill_kernel<<<nblk(32LL * b.n_wide, 128), 128, 0, s>>>(
@@ -1041,7 +1012,7 @@ static cudaError_t fill_wide(BvhBuffers& b, cudaStream_t s) {
 template <int DIM>
 static cudaError_t build_wide(BvhBuffers& b, cudaStream_t s) {
     constexpr int W = DIM == 2 ? kWide : kOriented;
-    constexpr int kNodeFloats = DIM == 2 ? WideLayout<2>::kFloats : 4 * kOrientedF4;
+    constexpr int kNodeFloats = DIM == 2 ? kWideFloats : 4 * kOrientedF4;
     constexpr int kMax = DIM == 2 ? (kWideStack - 1) / (kWide - 1) : kOrientedDepthMax;   // levels the search takes
     static_assert(kMax < kWideLevels, "level counts");
     const int n_int = b.n_internal;

@@ -470,23 +470,18 @@ __device__ __forceinline__ float gradient_factor(float k, float R) {
 }
 
 // ---- 32-wide BVH of segments, searched by a whole warp ----------------------
-// The binary LBVH collapsed five levels at a time: a wide node holds up to 32
-// children in SoA order, lo[DIM][32], hi[DIM][32], code[32] (>= 0: wide node,
-// < 0: ~leaf, kEmptyChild: unused slot with an empty box) and, for leaf
-// children, the element's vertices vtx[DIM * DIM][32] (segment a, b or
-// triangle a, b, c), so that lane j of a warp loads slot j of every array with
-// one coalesced request per array, and a visit needs one round trip to memory
-// whether its children are nodes or elements.
+// The binary LBVH collapsed five levels at a time: a wide node holds 32 child slots,
+// one per lane: a float4 (an inner child's box lo.xy hi.xy, or a leaf child's segment
+// a.xy b.xy, so that a visit needs one round trip to memory whether its children are
+// nodes or elements) and then 32 codes (>= 0: wide node, < 0: ~leaf, kEmptyChild:
+// unused slot); a warp reads either in one coalesced request.
 constexpr int kWide = 32;
 constexpr int kWideStack = 224;            // stack entries per warp: 31 x wide depth + 1 (checked at build): depth <= 7
 constexpr unsigned kWarpAll = 0xffffffffu;
-template <int DIM> struct WideLayout {
-    static constexpr int kVtx = (2 * DIM + 1) * kWide;              // offset of the vertex arrays
-    static constexpr int kFloats = (2 * DIM + 1 + DIM * DIM) * kWide;
-};
+constexpr int kWideFloats = 5 * kWide;     // floats of a node: the float4s, then the codes
 
 struct WideView {
-    const float* wnodes;   // n_wide nodes, root first (2D: WideLayout, 3D: oriented nodes)
+    const float* wnodes;   // n_wide nodes, root first (2D: kWideFloats floats, 3D: oriented nodes)
     const float4* prims;
     int n_wide;
     int n_tree;
@@ -495,18 +490,17 @@ struct WideView {
 
 // Closest tree leaf for every lane in `need`, one query at a time, with all
 // 32 lanes working on it: each lane takes one child slot of the current wide
-// node, leaf children are measured exactly in parallel and reduced with
-// shuffles (ties to the lower leaf index), and the inner children that can
-// still hold a closer leaf go on the warp's stack in shared memory with the
-// nearest on top (depth-first, nearest child first, the others in Morton
-// order, all pruned by the running bound when popped).  n_nodes counts node
+// node, leaf children are measured exactly in parallel and reduced to the minimum
+// (ties to the lower leaf index), the nearest inner child that can still hold a
+// closer leaf is visited next, and the others go on the warp's stack in shared memory
+// in Morton order (a pop looks at the top 32 entries at once for the first that
+// is still within the bound).  n_nodes counts node
 // visits (a leaf child's vertices come with its node).
 // best2 / best hold each lane's bound on entry (kInf / -1 without one) and
 // the result on exit.  Called by all 32 lanes with the same `need` and each
-// lane's own view (lanes may belong to different problems).  Returns error
-// bits: 1 if a query popped more nodes than the tree has, 4 if the stack
-// would overflow (excluded by the build's depth check).
-template <int DIM>
+// lane's own view (lanes may belong to different problems).  Returns 1 if a
+// query visited more nodes than its budget or the stack would overflow
+// (excluded by the build's depth check).
 __device__ __forceinline__ int wide_closest(const WideView& mine, unsigned need, const float* q_lane, float& best2,
                                             int& best, float2* stk, unsigned& n_nodes, unsigned& n_prims) {
     const int lane = threadIdx.x & 31;
@@ -514,86 +508,77 @@ __device__ __forceinline__ int wide_closest(const WideView& mine, unsigned need,
     while (need) {
         const int src = __ffs(need) - 1;
         need &= need - 1;
-        float q[DIM];
-#pragma unroll
-        for (int k = 0; k < DIM; ++k) q[k] = __shfl_sync(kWarpAll, q_lane[k], src);
+        const float q[2] = {__shfl_sync(kWarpAll, q_lane[0], src), __shfl_sync(kWarpAll, q_lane[1], src)};
         float b2 = __shfl_sync(kWarpAll, best2, src);
         int bi = __shfl_sync(kWarpAll, best, src);
         const float* wn = reinterpret_cast<const float*>(
             __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.wnodes), src));
-        const float4* prims = reinterpret_cast<const float4*>(
-            __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.prims), src));
         const int n_wide = __shfl_sync(kWarpAll, mine.n_wide, src);
-        const int n_tree = __shfl_sync(kWarpAll, mine.n_tree, src);
         const int cap = __shfl_sync(kWarpAll, mine.budget, src);
         if (n_wide > 0) {
-            __syncwarp();
-            if (lane == 0) stk[0] = make_float2(0.0f, __int_as_float(0));
-            __syncwarp();
-            int top = 1;
             int budget = cap > 0 ? cap : n_wide;
-            while (top > 0) {
-                const float2 e = stk[top - 1];
-                --top;
-                if (!within(e.x, b2)) continue;                // pruned by a closer leaf found since
-                if (--budget < 0) { err |= 1; break; }
-                const float* f = wn + (size_t)__float_as_int(e.y) * WideLayout<DIM>::kFloats;
-                float lo[DIM], hi[DIM], vt[DIM * DIM];
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) {
-                    lo[k] = __ldg(f + k * kWide + lane);
-                    hi[k] = __ldg(f + (DIM + k) * kWide + lane);
-                }
-                const int code = __float_as_int(__ldg(f + 2 * DIM * kWide + lane));
-#pragma unroll
-                for (int k = 0; k < DIM * DIM; ++k) vt[k] = __ldg(f + WideLayout<DIM>::kVtx + k * kWide + lane);
-                const float cd = box_dist2<DIM>(q, lo, hi);
+            int top = 0, cur = 0;
+            for (;;) {
+                if (--budget < 0) { err = 1; break; }
+                const float* f = wn + (size_t)cur * kWideFloats;
+                const float4 s = __ldg(reinterpret_cast<const float4*>(f) + lane);
+                const int code = __float_as_int(__ldg(f + 4 * kWide + lane));
                 if (lane == 0) ++n_nodes;
-                const bool leaf = code < 0 && within(cd, b2);
-                const unsigned lm = __ballot_sync(kWarpAll, leaf);
-                if (lm) {
-                    float dd = kInf;
-                    if (leaf) {
-                        if (DIM == 2) {
-                            float t;
-                            dd = seg_closest(q, vt[0], vt[1], vt[2], vt[3], t);
-                        } else {
-                            float w1, w2;
-                            dd = tri_closest(q, make_float3(vt[0], vt[1], vt[2]), make_float3(vt[3], vt[4], vt[5]),
-                                             make_float3(vt[6], vt[7], vt[8]), w1, w2);
-                        }
-                    }
+                if (__any_sync(kWarpAll, code < 0)) {
+                    float t, dd = kInf;
+                    if (code < 0) dd = seg_closest(q, s.x, s.y, s.z, s.w, t);
                     // warp argmin, ties to the lower leaf index: squared distances are >= 0 (or
                     // +inf), so their bit patterns order like the values and one integer
                     // reduction finds the minimum; a second one picks the tied leaf
                     const unsigned bits = __float_as_uint(dd);
                     const unsigned mbits = __reduce_min_sync(kWarpAll, bits);
-                    const unsigned pi = __reduce_min_sync(kWarpAll, leaf && bits == mbits ? (unsigned)~code : 0xffffffffu);
                     const float md = __uint_as_float(mbits);
-                    if (closer(md, (int)pi, b2, bi)) { b2 = md; bi = (int)pi; }
+                    if (md <= b2) {
+                        const unsigned pi = __reduce_min_sync(kWarpAll, code < 0 && bits == mbits ? (unsigned)~code : 0xffffffffu);
+                        if (closer(md, (int)pi, b2, bi)) { b2 = md; bi = (int)pi; }
+                    }
                 }
+                const float lo[2] = {s.x, s.y}, hi[2] = {s.z, s.w};
+                const float cd = box_dist2<2>(q, lo, hi);
                 const bool inner = code >= 0 && code != kEmptyChild && within(cd, b2);
                 const unsigned im = __ballot_sync(kWarpAll, inner);
                 if (im) {
-                    const int cnt = __popc(im);
-                    if (top + cnt > kWideStack) { err |= 4; break; }
-                    // the nearest child (ties to the lower lane) goes on top (popped next); its
-                    // siblings below it in lane order, which is the Morton order of the subtrees
-                    const unsigned cbits = inner ? __float_as_uint(cd) : 0xffffffffu;
-                    const unsigned mc = __reduce_min_sync(kWarpAll, cbits);
-                    const int ml = __ffs(__ballot_sync(kWarpAll, inner && cbits == mc)) - 1;
-                    const unsigned rest = im & ~(1u << ml);
-                    __syncwarp();
-                    if (inner) {
-                        const int pos = lane == ml ? cnt - 1 : __popc(rest & ((1u << lane) - 1u));
-                        stk[top + pos] = make_float2(cd, __int_as_float(code));
+                    // the nearest child (the low bits of its distance give way to its lane) is next
+                    const int cnt = __popc(im) - 1;
+                    if (top + cnt > kWideStack) { err = 1; break; }
+                    int ml = __ffs(im) - 1;
+                    if (cnt > 0) {
+                        const unsigned key = inner ? (__float_as_uint(cd) & ~31u) | (unsigned)lane : 0xffffffffu;
+                        ml = (int)(__reduce_min_sync(kWarpAll, key) & 31u);
+                        const unsigned rest = im & ~(1u << ml);
+                        __syncwarp();
+                        if (inner && lane != ml)
+                            stk[top + __popc(rest & ((1u << lane) - 1u))] = make_float2(cd, __int_as_float(code));
+                        top += cnt;
+                        __syncwarp();
                     }
-                    top += cnt;
-                    __syncwarp();
+                    cur = __shfl_sync(kWarpAll, code, ml);
+                    continue;
                 }
+                // pop the topmost entry that is still within the bound
+                unsigned ok = 0;
+                float2 e = make_float2(kInf, 0.0f);
+                while (top > 0) {
+                    const int at = top - 1 - lane;
+                    if (at >= 0) e = stk[at];
+                    ok = __ballot_sync(kWarpAll, at >= 0 && within(e.x, b2));
+                    if (ok) break;
+                    top = max(top - 32, 0);
+                }
+                if (!ok) break;
+                const int first = __ffs(ok) - 1;
+                cur = __shfl_sync(kWarpAll, __float_as_int(e.y), first);
+                top -= 1 + first;
             }
-        } else if (n_tree == 1) {
-            const float dd = prim_dist2<DIM>(prims, 0, q);
+        } else if (__shfl_sync(kWarpAll, mine.n_tree, src) == 1) {
+            const float4* prims = reinterpret_cast<const float4*>(
+                __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.prims), src));
+            const float dd = prim_dist2<2>(prims, 0, q);
             if (lane == 0) ++n_prims;
             if (closer(dd, 0, b2, bi)) { b2 = dd; bi = 0; }
         }
@@ -863,7 +848,7 @@ __host__ __device__ inline size_t wide_smem_bytes(int dim, int stk_cap) {   // p
 template <int DIM>
 __device__ __forceinline__ int wide_search(const WideView& mine, unsigned need, const float* q, float& best2, int& best,
                                            float2* stk, int stk_cap, unsigned& n_nodes, unsigned& n_prims) {
-    if constexpr (DIM == 2) return wide_closest<DIM>(mine, need, q, best2, best, stk, n_nodes, n_prims);
+    if constexpr (DIM == 2) return wide_closest(mine, need, q, best2, best, stk, n_nodes, n_prims);
     else return oriented_closest(mine, need, q, best2, best, reinterpret_cast<SearchScratch*>(stk), stk_cap, n_nodes, n_prims);
 }
 

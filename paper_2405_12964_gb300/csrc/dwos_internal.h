@@ -150,7 +150,7 @@ struct BvhBuffers {
     size_t sort_tmp_bytes = 0;
     int capacity = 0;
     // wide tree collapsed from the binary one (rebuilt with it), nodes level by level
-    float* wnodes = nullptr;         // n_wide nodes (2D WideLayout, 3D kOrientedF4 float4)
+    float* wnodes = nullptr;         // n_wide nodes (2D kWideFloats floats, 3D kOrientedF4 float4)
     int* wsrc = nullptr;             // per slot: (binary parent << 1 | side) of the child's box, -1 unused; then per
                                      // slot its code; then per node the slot that holds it
     int* wroot = nullptr;            // per wide node: the binary node it was collapsed from; then the id of its
