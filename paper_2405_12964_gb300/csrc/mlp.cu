@@ -2,10 +2,15 @@
 // -> 4 x 64 tanh -> 8 linear outputs (0: u, 1: du/dn), trained and evaluated
 // on the 5th-generation tensor cores.
 //
-// One persistent kernel (256 threads, one CTA per SM) walks over tiles of 128
-// samples; sample row r is TMEM lane r, and threads r and r + 128 share it
-// (warps w and w + 4 reach the same TMEM lane quarter): each takes half of the
-// row's columns in the epilogues between the products.  Operands
+// One persistent kernel (512 threads, one CTA per SM) walks over tiles of 128
+// samples; sample row r is TMEM lane r, and threads r, r + 128, r + 256 and r + 384
+// share it (warps w, w + 4, ... reach the same TMEM lane quarter): each takes 16 of the
+// row's 64 columns in the epilogues between the products.  The ten products of a tile
+// are a chain (each operand is the last product's epilogue), so a CTA's time is the
+// chain's latency: four threads to a row instead of two halve the issue time of the
+// tanh epilogues, each link has one block barrier, and the weight gradients of a layer
+// run while the threads work on the next layer's deltas (two delta tiles in turn).
+// Operands
 // live in shared memory as BF16 in the canonical no-swizzle core-matrix
 // layout (8 rows x 16 bytes per 128-byte core matrix), the products are
 // tcgen05.mma (kind::f16, BF16 in, FP32 accumulate) issued by one thread and
@@ -38,7 +43,7 @@ constexpr int OUT = 8;           // output width
 constexpr int OUTP = 16;         // output rows padded for the N = 16 product
 constexpr int NP = DWOS_MLP_NPARAM;
 constexpr int TILE = 128;        // samples per tile (the MMA's M)
-constexpr int THREADS = 256;          // two threads per sample row
+constexpr int THREADS = 512;          // four threads per sample row
 // offsets of W_l and b_l (l = 1..5) in the flat parameter vector
 __host__ __device__ constexpr int off_w(int l) { return l == 1 ? 0 : 1088 + (l - 2) * 4160; }
 __host__ __device__ constexpr int off_b(int l) { return l == 1 ? 1024 : (l == 5 ? 14080 : 1088 + (l - 2) * 4160 + 4096); }
@@ -68,7 +73,7 @@ struct __align__(1024) Smem {
     WImage w;                                   // 28672 B
     __nv_bfloat16 a0[TILE * C0];                // 8 KB
     __nv_bfloat16 a[4][TILE * CA];              // 4 x 20 KB
-    __nv_bfloat16 d[TILE * CD];                 // 32 KB
+    __nv_bfloat16 d[2][TILE * CD];              // 2 x 32 KB: delta_l in d[l & 1]
     float bias[4 * H + OUT];
     unsigned long long bar_load, bar_mma;
     uint32_t tmem_base;
@@ -192,8 +197,8 @@ __device__ __forceinline__ void feats(float x, float y, float* f) {
 
 enum Mode { kTrain = 0, kEval = 1 };
 
-// mode kTrain: masked-MSE loss (sum over this CTA's samples, FP64, one atomic
-// per warp) and the CTA's gradient partial (NP floats at part + blockIdx.x * NP).
+// mode kTrain: masked-MSE loss (sums of this CTA's four warps of rows at loss + 4 *
+// blockIdx.x) and the CTA's gradient partial (NP floats at part + blockIdx.x * NP).
 // mode kEval: u, d u / d (x, y) and du/dn per sample.
 template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
@@ -205,7 +210,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     Smem& S = *reinterpret_cast<Smem*>(raw);
     const int tid = threadIdx.x;
     const int r = tid & (TILE - 1);            // sample row and TMEM lane
-    const int half = tid >> 7;                 // which half of the row's columns this thread takes
+    const int q16 = tid >> 7;                  // which 16 of the row's columns this thread takes
     const int warp = tid >> 5;
     const uint32_t bar_load = smem_u32(&S.bar_load), bar_mma = smem_u32(&S.bar_mma);
     if (tid == 0) {
@@ -213,8 +218,11 @@ __global__ void __launch_bounds__(THREADS, 1)
         bar_init(bar_mma, 1);
         S.fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        bar_expect_tx(bar_load, sizeof(WImage));
+        bulk_g2s(smem_u32(&S.w), wimg, sizeof(WImage), bar_load);
     }
     if (warp == 0) {
+        __syncwarp();
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :: "r"(smem_u32(&S.tmem_base)), "r"(TMEM_COLS));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
@@ -225,27 +233,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     {
         const float z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         const float one[8] = {1, 0, 0, 0, 0, 0, 0, 0};
-        if (half == 0) {
+        if (q16 == 0) {
+            put8(S.a0, C0, r, 1, z);
             put8(S.a0, C0, r, 2, one);
             put8(S.a0, C0, r, 3, z);
-            for (int l = 0; l < 4; ++l) {
-                put8(S.a[l], CA, r, 8, one);
-                put8(S.a[l], CA, r, 9, z);
-            }
         }
-        for (int cc = half * (CD / 16); cc < (half + 1) * (CD / 16); ++cc) put8(S.d, CD, r, cc, z);
+        put8(S.a[q16], CA, r, 8, one);
+        put8(S.a[q16], CA, r, 9, z);
+        for (int cc = q16; cc < CD / 8; cc += 4) {
+            put8(S.d[0], CD, r, cc, z);
+            put8(S.d[1], CD, r, cc, z);
+        }
     }
     fence_before();
     __syncthreads();
     fence_after();
     const uint32_t tmem = S.tmem_base;
     const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);   // this warp's TMEM lane quarter
-    if (tid == 0) {
-        bar_expect_tx(bar_load, sizeof(WImage));
-        bulk_g2s(smem_u32(&S.w), wimg, sizeof(WImage), bar_load);
-    }
-    bool ok = bar_wait(bar_load, 0);
-    ok = !__syncthreads_or(!ok);
+    bool ok = bar_wait(bar_load, 0);   // agreed on by the next publish()
     uint32_t phase = 0;
     const __nv_bfloat16* W[6] = {nullptr, S.w.w1, S.w.w2, S.w.w3, S.w.w4, S.w.w5};
     const int CW[6] = {0, IN, H, H, H, H};     // columns of W_l (its K in the forward product)
@@ -253,80 +258,91 @@ __global__ void __launch_bounds__(THREADS, 1)
     float loss_acc = 0.0f;
     const int n_tiles = (n + TILE - 1) / TILE;
 
-    // thread 0 commits the issued products; everyone waits; false if any wait failed
-    auto sync_mma = [&]() -> bool {
-        if (tid == 0) mma_commit(bar_mma);
-        const bool got = bar_wait(bar_mma, phase);
+    // Everyone waits for the products thread 0 committed; a wait that runs out clears ok,
+    // which the next publish() makes the whole block's.
+    auto wait_mma = [&]() {
+        ok = bar_wait(bar_mma, phase) && ok;
         phase ^= 1u;
+        __syncwarp();
         fence_after();
-        return !__syncthreads_or(!got);
     };
-    auto publish = [&]() {     // smem written by the threads -> visible to the next products
+    // smem written by the threads -> visible to the next products; ok of all threads
+    auto publish = [&]() {
         fence_async_smem();
         fence_before();
-        __syncthreads();
+        ok = !__syncthreads_or(!ok);
         fence_after();
+    };
+    // a tile's sample of this row, its features and training target (the threads of columns 0..15)
+    float px = 0.0f, py = 0.0f, f[8];
+    float2 tg = make_float2(0.0f, 0.0f), mk = tg;
+    auto load_sample = [&](int tile) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) f[i] = 0.0f;
+        if (q16 != 0 || tile >= n_tiles) return;
+        const int s = tile * TILE + r;
+        if (s >= n) return;
+        px = x[2 * s];
+        py = x[2 * s + 1];
+        if (MODE == kTrain) {
+            tg = make_float2(target[2 * s], target[2 * s + 1]);
+            mk = make_float2(mask[2 * s], mask[2 * s + 1]);
+        }
+        feats(px, py, f);
     };
 
     int tiles_done = 0;
-    for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x, ++tiles_done) {
+    load_sample(blockIdx.x);
+    for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tiles_done) {
         const int s = tile * TILE + r;
         const bool valid = s < n;
-        float px = 0.0f, py = 0.0f;
-        if (valid) { px = x[2 * s]; py = x[2 * s + 1]; }
-        if (half == 0) {
-            float f[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            if (valid) feats(px, py, f);
-            const float z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-            put8(S.a0, C0, r, 0, f);
-            put8(S.a0, C0, r, 1, z);
-        }
+        if (q16 == 0) put8(S.a0, C0, r, 0, f);
         publish();
+        if (!ok) break;
         // ---- forward: four tanh layers
-        for (int l = 1; l <= 4 && ok; ++l) {
+        for (int l = 1; l <= 4; ++l) {
             const __nv_bfloat16* A = l == 1 ? S.a0 : S.a[l - 2];
             const int CAin = l == 1 ? C0 : CA;
             if (tid == 0) {
-                fence_after();
                 for (int ks = 0; ks < CW[l] / 16; ++ks)
                     mma(tmem + T_SCR, kmajor(A, CAin, ks), kmajor(W[l], CW[l], ks), idesc_bf16(128, 64, false, false),
                         ks > 0 ? 1u : 0u);
+                mma_commit(bar_mma);
             }
-            ok = sync_mma();
-            if (!ok) break;
-            for (int c16 = 2 * half; c16 < 2 * half + 2; ++c16) {
-                float v[16];
-                tmem_ld16(lane_addr + T_SCR + 16 * c16, v);
+            wait_mma();
+            float v[16];
+            tmem_ld16(lane_addr + T_SCR + 16 * q16, v);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] = tanhf(v[i] + S.bias[(l - 1) * H + 16 * c16 + i]);
-                put8(S.a[l - 1], CA, r, 2 * c16, v);
-                put8(S.a[l - 1], CA, r, 2 * c16 + 1, v + 8);
-            }
+            for (int i = 0; i < 16; ++i) v[i] = tanhf(v[i] + S.bias[(l - 1) * H + 16 * q16 + i]);
+            put8(S.a[l - 1], CA, r, 2 * q16, v);
+            put8(S.a[l - 1], CA, r, 2 * q16 + 1, v + 8);
             publish();
+            if (!ok) break;
         }
         if (!ok) break;
         // ---- output layer
         if (tid == 0) {
-            fence_after();
             for (int ks = 0; ks < 4; ++ks)
                 mma(tmem + T_SCR, kmajor(S.a[3], CA, ks), kmajor(S.w.w5, H, ks), idesc_bf16(128, 16, false, false),
                     ks > 0 ? 1u : 0u);
+            mma_commit(bar_mma);
         }
-        ok = sync_mma();
-        if (!ok) break;
-        if (half == 0) {
+        wait_mma();
+        if (q16 == 0) {
             float o[16];
             tmem_ld16(lane_addr + T_SCR, o);
             float d5[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) d5[i] = 0.0f;
             if (MODE == kTrain) {
-                if (valid)
+                if (valid) {
+                    const float t2[2] = {tg.x, tg.y}, m2[2] = {mk.x, mk.y};
                     for (int k = 0; k < 2; ++k) {
-                        const float e = mask[2 * s + k] * (o[k] + S.bias[4 * H + k] - target[2 * s + k]);
+                        const float e = m2[k] * (o[k] + S.bias[4 * H + k] - t2[k]);
                         loss_acc += e * e;
                         d5[k] = 2.0f * e * inv_n;
                     }
+                }
             } else {
                 if (valid) {
                     if (u_out) u_out[s] = o[0] + S.bias[4 * H];
@@ -334,78 +350,86 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
                 d5[0] = 1.0f;        // d u / d out
             }
-            put8(S.d, CD, r, 0, d5);
-            put8(S.d, CD, r, 1, d5 + 8);
+            put8(S.d[1], CD, r, 0, d5);
+            put8(S.d[1], CD, r, 1, d5 + 8);
         }
         publish();
-        // ---- backward: weight gradients (training) and the deltas
-        for (int l = 5; l >= 1 && ok; --l) {
+        if (!ok) break;
+        // ---- backward: the deltas, and weight gradients (training).  Layer l's weight
+        // gradient is issued after its delta product was committed: the wait on that product
+        // covers layer l + 1's weight gradient, which read the delta tile written next.
+        for (int l = 5; l >= 1; --l) {
             const __nv_bfloat16* Ain = l == 1 ? S.a0 : S.a[l - 2];
+            const __nv_bfloat16* D = S.d[l & 1];
             const int CAin = l == 1 ? C0 : CA;
             const bool delta_product = l > 1 || MODE == kEval;
             if (tid == 0) {
-                fence_after();
-                if (MODE == kTrain)
-                    for (int ks = 0; ks < TILE / 16; ++ks)
-                        mma(tmem + t_dw(l), mnmajor(S.d, CD, ks), mnmajor(Ain, CAin, ks),
-                            idesc_bf16(128, CAin, true, true), (tiles_done > 0 || ks > 0) ? 1u : 0u);
                 if (delta_product) {
                     const int kout = l == 5 ? OUTP : H;  // K of the product: layer l's outputs
                     const int nin = l == 1 ? IN : H;     // N: its inputs
                     for (int ks = 0; ks < kout / 16; ++ks)
-                        mma(tmem + T_SCR, kmajor(S.d, CD, ks), mnmajor(W[l], CW[l], ks),
+                        mma(tmem + T_SCR, kmajor(D, CD, ks), mnmajor(W[l], CW[l], ks),
                             idesc_bf16(128, nin, false, true), ks > 0 ? 1u : 0u);
+                    mma_commit(bar_mma);
+                }
+                if (MODE == kTrain) {
+                    for (int ks = 0; ks < TILE / 16; ++ks)
+                        mma(tmem + t_dw(l), mnmajor(D, CD, ks), mnmajor(Ain, CAin, ks),
+                            idesc_bf16(128, CAin, true, true), (tiles_done > 0 || ks > 0) ? 1u : 0u);
+                    if (l == 1) mma_commit(bar_mma);
                 }
             }
-            ok = sync_mma();
-            if (!ok) break;
+            if (MODE == kTrain && l == 1) load_sample(tile + gridDim.x);   // while the last products run
+            wait_mma();
             if (l > 1) {
                 // delta_{l-1} = (delta_l W_l) * (1 - a_{l-1}^2), a as stored (BF16)
-                for (int c16 = 2 * half; c16 < 2 * half + 2; ++c16) {
-                    float v[16], a[16];
-                    tmem_ld16(lane_addr + T_SCR + 16 * c16, v);
-                    get8(S.a[l - 2], CA, r, 2 * c16, a);
-                    get8(S.a[l - 2], CA, r, 2 * c16 + 1, a + 8);
+                float v[16], a[16];
+                tmem_ld16(lane_addr + T_SCR + 16 * q16, v);
+                get8(S.a[l - 2], CA, r, 2 * q16, a);
+                get8(S.a[l - 2], CA, r, 2 * q16 + 1, a + 8);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] *= 1.0f - a[i] * a[i];
-                    put8(S.d, CD, r, 2 * c16, v);
-                    put8(S.d, CD, r, 2 * c16 + 1, v + 8);
-                }
+                for (int i = 0; i < 16; ++i) v[i] *= 1.0f - a[i] * a[i];
+                put8(S.d[(l - 1) & 1], CD, r, 2 * q16, v);
+                put8(S.d[(l - 1) & 1], CD, r, 2 * q16 + 1, v + 8);
                 publish();
+                if (!ok) break;
             } else if (MODE == kEval) {
                 float df[16];
-                if (half == 0) tmem_ld16(lane_addr + T_SCR, df);       // d u / d features
-                if (half == 0 && valid && g_out) {
+                if (q16 == 0) tmem_ld16(lane_addr + T_SCR, df);       // d u / d features
+                if (q16 == 0 && valid && g_out) {
                     const float c0 = 3.14159265358979f * cospif(px), c1 = 3.14159265358979f * cospif(py);
                     const float c01 = 3.14159265358979f * cospif(px + py);
                     g_out[2 * s] = df[0] + df[2] * c0 + df[4] * c01;
                     g_out[2 * s + 1] = df[1] + df[3] * c1 + df[4] * c01;
                 }
-                fence_before();
-                __syncthreads();
-                fence_after();
+                load_sample(tile + gridDim.x);
             }
         }
     }
+    // ok after the last products of the last tile, and every thread's reads of TMEM before them
+    fence_before();
+    ok = !__syncthreads_or(!ok);
+    fence_after();
 
     if (MODE == kTrain && ok) {
         for (int off = 16; off > 0; off >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, off);
-        if ((tid & 31) == 0 && loss_acc != 0.0f) atomicAdd(loss, (double)loss_acc * (double)inv_n);
+        if ((tid & 31) == 0 && q16 == 0) loss[4 * blockIdx.x + warp] = (double)loss_acc * (double)inv_n;
         // the CTA's weight and bias gradients: rows (outputs) are TMEM lanes 0..63
         float* P = part + (size_t)blockIdx.x * NP;
         for (int l = 1; l <= 5; ++l) {
             const int outs = l == 5 ? OUT : H, ins = l == 1 ? IN : H;
             const int ncol = l == 1 ? C0 : CA;
-            for (int c16 = half; c16 < ncol / 16; c16 += 2) {
+            for (int c16 = q16; c16 < ncol / 16; c16 += 4) {
                 float v[16];
+                __syncwarp();
                 tmem_ld16(lane_addr + t_dw(l) + 16 * c16, v);     // warp-wide: every warp loads
-                if (r < outs)
+                if (r < outs && 16 * c16 < ins) {
+                    float4* o = reinterpret_cast<float4*>(P + off_w(l) + r * ins + 16 * c16);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const int c = 16 * c16 + i;
-                        if (c < ins) P[off_w(l) + r * ins + c] = v[i];
-                        else if (c == ins) P[off_b(l) + r] = v[i];
-                    }
+                    for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                } else if (r < outs) {
+                    P[off_b(l) + r] = v[0];
+                }
             }
         }
     }
@@ -434,15 +458,6 @@ __global__ void wait_probe_kernel(int polls, int* __restrict__ err) {
     if (threadIdx.x == 0) atomicOr(err, 1);
 }
 
-// Sum of the CTA partials, in CTA order (deterministic).
-__global__ void reduce_parts_kernel(const float* __restrict__ part, int n_parts, float* __restrict__ grad) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= NP) return;
-    float s = 0.0f;
-    for (int c = 0; c < n_parts; ++c) s += part[(size_t)c * NP + i];
-    grad[i] = s;
-}
-
 // BF16 weight image in the shared-memory layout.
 __global__ void convert_kernel(const float* __restrict__ p, WImage* __restrict__ w) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -462,17 +477,53 @@ __global__ void convert_kernel(const float* __restrict__ p, WImage* __restrict__
     }
 }
 
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float gi = g[i];
+// Sums the CTA partials (gradient and loss, in CTA order: deterministic); with ADAM
+// it also takes the step and writes the new weights' BF16 image, so that a training step
+// is two launches.  Bound by the latency of the partials' loads (8.6 MB from L2): small
+// blocks spread them over all SMs, sixteen loads in flight per thread.
+constexpr int kUpdateThreads = 64;
+
+template <bool ADAM>
+__global__ void __launch_bounds__(kUpdateThreads) update_kernel(const float* __restrict__ part, int n_parts,
+                                                                const double* __restrict__ loss_part,
+                                                                float* __restrict__ g, double* __restrict__ loss,
+                                                                float* __restrict__ p, float* __restrict__ m,
+                                                                float* __restrict__ v, WImage* __restrict__ w,
+                                                                float lr, float b1, float b2, float eps, float c1,
+                                                                float c2) {
+    const int i = blockIdx.x * kUpdateThreads + threadIdx.x;
+    if (loss && blockIdx.x == 0 && threadIdx.x < 32) {
+        double s = 0.0;
+        for (int c = threadIdx.x; c < 4 * n_parts; c += 32) s += loss_part[c];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (threadIdx.x == 0) *loss = s;
+    }
+    if (i >= NP) return;
+    float gi = 0.0f;
+    int c = 0;
+    for (; c + 16 <= n_parts; c += 16) {
+        float t[16];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) t[k] = part[(size_t)(c + k) * NP + i];
+#pragma unroll
+        for (int k = 0; k < 16; ++k) gi += t[k];
+    }
+    for (; c < n_parts; ++c) gi += part[(size_t)c * NP + i];
+    g[i] = gi;
+    if (!ADAM) return;
     const float mi = b1 * m[i] + (1.0f - b1) * gi;
     const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+    const __nv_bfloat16 b = __float2bfloat16_rn(pi);
+    if (i < off_b(1)) { w->w1[core_off(i / IN, i % IN, IN)] = b; return; }
+    if (i < off_w(2)) return;
+    const int l = i < off_w(5) ? 2 + (i - off_w(2)) / 4160 : 5, j = i - off_w(l);
+    if (i >= off_b(l)) return;
+    __nv_bfloat16* wl = l == 2 ? w->w2 : l == 3 ? w->w3 : l == 4 ? w->w4 : w->w5;
+    wl[core_off(j / H, j % H, H)] = b;
 }
 
 }  // namespace
@@ -488,6 +539,7 @@ struct dwos_mlp {
     double* loss = nullptr;
     WImage* w = nullptr;         // BF16 weight image
     float* part = nullptr;       // per-CTA gradient partials (n_sm x NP)
+    double* loss_part = nullptr; // per-CTA loss partials (n_sm x 4)
     int* dflag = nullptr;        // device flag: a bounded wait ran out
     int n_sm = 0;
     float* scratch = nullptr;    // staging for host inputs
@@ -551,16 +603,15 @@ dwos_status check_err(dwos_mlp* mlp) {
     return DWOS_OK;
 }
 
-dwos_status grads(dwos_mlp* mlp, int n, const float* x, const float* t, const float* mk) {
-    MK(cudaMemsetAsync(mlp->loss, 0, sizeof(double), mlp->stream), "zero loss");
-    const int grid = grid_for(mlp, n);
-    mlp_kernel<kTrain><<<grid, THREADS, sizeof(Smem), mlp->stream>>>(mlp->w, mlp->p, n, x, t, mk, mlp->part,
-                                                                     mlp->loss, nullptr, nullptr, nullptr, mlp->dflag);
+// The training kernel: gradient and loss partials of the grid's CTAs.
+dwos_status launch_train(dwos_mlp* mlp, int n, const float* x, const float* t, const float* mk) {
+    mlp_kernel<kTrain><<<grid_for(mlp, n), THREADS, sizeof(Smem), mlp->stream>>>(
+        mlp->w, mlp->p, n, x, t, mk, mlp->part, mlp->loss_part, nullptr, nullptr, nullptr, mlp->dflag);
     MK(cudaGetLastError(), "train kernel");
-    reduce_parts_kernel<<<(NP + 255) / 256, 256, 0, mlp->stream>>>(mlp->part, grid, mlp->g);
-    MK(cudaGetLastError(), "reduce");
     return DWOS_OK;
 }
+
+constexpr int kUpdateBlocks = (NP + kUpdateThreads - 1) / kUpdateThreads;
 
 }  // namespace
 
@@ -580,6 +631,7 @@ dwos_status dwos_mlp_create(dwos_mlp** out, int device) {
     if (e == cudaSuccess) e = cudaMalloc(&mlp->w, sizeof(WImage));
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&mlp->n_sm, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMalloc(&mlp->part, sizeof(float) * NP * (size_t)(mlp->n_sm > 0 ? mlp->n_sm : 1));
+    if (e == cudaSuccess) e = cudaMalloc(&mlp->loss_part, sizeof(double) * 4 * (size_t)(mlp->n_sm > 0 ? mlp->n_sm : 1));
     if (e == cudaSuccess) e = cudaMalloc(&mlp->dflag, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(mlp->dflag, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(mlp->w, 0, sizeof(WImage));
@@ -605,7 +657,7 @@ void dwos_mlp_destroy(dwos_mlp* mlp) {
     cudaSetDevice(mlp->device);
     if (mlp->stream) cudaStreamSynchronize(mlp->stream);
     for (void* p : {(void*)mlp->p, (void*)mlp->g, (void*)mlp->m, (void*)mlp->v, (void*)mlp->loss, (void*)mlp->w,
-                    (void*)mlp->scratch, (void*)mlp->part, (void*)mlp->dflag})
+                    (void*)mlp->scratch, (void*)mlp->part, (void*)mlp->loss_part, (void*)mlp->dflag})
         if (p) cudaFree(p);
     delete mlp;
 }
@@ -650,7 +702,11 @@ dwos_status dwos_mlp_loss_grad(dwos_mlp* mlp, int n, const float* x, const float
     const float* in[3] = {x, target, mask};
     float* d[3];
     if (dwos_status s = stage(mlp, mem, 2 * (size_t)n, in, d, 3)) return s;
-    if (dwos_status s = grads(mlp, n, d[0], d[1], d[2])) return s;
+    if (dwos_status s = launch_train(mlp, n, d[0], d[1], d[2])) return s;
+    update_kernel<false><<<kUpdateBlocks, kUpdateThreads, 0, mlp->stream>>>(
+        mlp->part, grid_for(mlp, n), mlp->loss_part, mlp->g, mlp->loss, nullptr, nullptr, nullptr, nullptr, 0.0f, 0.0f,
+        0.0f, 0.0f, 0.0f, 0.0f);
+    MK(cudaGetLastError(), "reduce");
     const cudaMemcpyKind k = mem == DWOS_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (grad) MK(cudaMemcpyAsync(grad, mlp->g, sizeof(float) * NP, k, mlp->stream), "copy grad");
     if (loss) MK(cudaMemcpyAsync(loss, mlp->loss, sizeof(double), k, mlp->stream), "copy loss");
@@ -666,18 +722,17 @@ dwos_status dwos_mlp_train_step(dwos_mlp* mlp, int n, const float* x, const floa
     const float* in[3] = {x, target, mask};
     float* d[3];
     if (dwos_status s = stage(mlp, mem, 2 * (size_t)n, in, d, 3)) return s;
-    if (dwos_status s = grads(mlp, n, d[0], d[1], d[2])) return s;
+    if (dwos_status s = launch_train(mlp, n, d[0], d[1], d[2])) return s;
     mlp->step += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - powf(b1, (float)mlp->step), c2 = 1.0f - powf(b2, (float)mlp->step);
-    adam_kernel<<<(NP + 255) / 256, 256, 0, mlp->stream>>>(mlp->p, mlp->g, mlp->m, mlp->v, NP, lr, b1, b2, 1e-8f,
-                                                           c1, c2);
-    MK(cudaGetLastError(), "adam");
-    convert_kernel<<<(H * H + 255) / 256, 256, 0, mlp->stream>>>(mlp->p, mlp->w);
-    MK(cudaGetLastError(), "convert");
-    if (loss) MK(cudaMemcpyAsync(loss, mlp->loss, sizeof(double),
-                                 mem == DWOS_MEM_DEVICE ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                                 mlp->stream), "copy loss");
+    double* d_loss = loss && mem == DWOS_MEM_DEVICE ? loss : mlp->loss;
+    update_kernel<true><<<kUpdateBlocks, kUpdateThreads, 0, mlp->stream>>>(
+        mlp->part, grid_for(mlp, n), mlp->loss_part, mlp->g, d_loss, mlp->p, mlp->m, mlp->v, mlp->w, lr, b1, b2, 1e-8f,
+        c1, c2);
+    MK(cudaGetLastError(), "update");
+    if (loss && mem != DWOS_MEM_DEVICE)
+        MK(cudaMemcpyAsync(loss, mlp->loss, sizeof(double), cudaMemcpyDeviceToHost, mlp->stream), "copy loss");
     if (mem == DWOS_MEM_HOST) return check_err(mlp);
     return DWOS_OK;
 }
