@@ -990,15 +990,15 @@ dwos_status dwos_eval(dwos_ctx* ctx, int n_query, const float* xq, int W, double
     CK(grow(ctx->out, ctx->out_cap, need), "alloc outputs");
     double* m = mem == DWOS_MEM_DEVICE ? u_mean : ctx->out;
     double* se = mem == DWOS_MEM_DEVICE ? u_se : ctx->out + n_query;
-    CK(launch_reduce_u(ctx->rec, n_query, W, m, se, ctx->stream), "reduce u");
-    ctx->launches += n_query > 0 ? 1 : 0;
-    if (diff) {
+    if (!diff) {
+        CK(launch_reduce_u(ctx->rec, n_query, W, m, se, ctx->stream), "reduce u");
+    } else {
         double* dm = mem == DWOS_MEM_DEVICE ? du_mean : ctx->out + 2 * (size_t)n_query;
         double* ds = mem == DWOS_MEM_DEVICE ? du_se : ctx->out + 2 * (size_t)n_query + (size_t)n_query * N;
-        CK(launch_reduce_udot(ctx->rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, N, n_query, W, dm, ds,
+        CK(launch_reduce_udot(ctx->rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, N, n_query, W, m, se, dm, ds,
                               ctx->stream), "reduce udot");
-        ctx->launches += n_query > 0 ? 1 : 0;
     }
+    ctx->launches += n_query > 0 ? 1 : 0;
     if (mem == DWOS_MEM_HOST) {
         CK(from_device(ctx, u_mean, ctx->out, n_query, mem), "copy u");
         CK(from_device(ctx, u_se, ctx->out + n_query, n_query, mem), "copy se");
@@ -1187,13 +1187,11 @@ dwos_status dwos_grad_l2_cv(dwos_ctx* ctx, int n_query, const float* xq, const f
     CK(grow(ctx->out, ctx->out_cap, 2 * (size_t)n_query), "alloc outputs");
     double* mean = ctx->out;
     double* se = ctx->out + n_query;
-    CK(launch_reduce_u(ctx->rec, n_query, W, mean, se, ctx->stream, cvp), "reduce u");
+    // u_var: per-point standard errors without and with the control variate
+    CK(launch_reduce_u(ctx->rec, n_query, W, mean, u_var ? u_var + n_query : se, ctx->stream, cvp, 0, u_var),
+       "reduce u");
     CK(launch_loss(mean, ctx->wvec, n_query, loss, ctx->stream), "loss");
-    if (u_var) {   // per-point standard errors without and with the control variate
-        CK(launch_reduce_u(ctx->rec, n_query, W, mean, u_var, ctx->stream, nullptr), "reduce u");
-        CK(launch_reduce_u(ctx->rec, n_query, W, mean, u_var + n_query, ctx->stream, cvp), "reduce u");
-    }
-    ctx->launches += 4 + (N > 0) + (u_var ? 2 : 0);
+    ctx->launches += 4 + (N > 0);
     if (samples) {
         CK(launch_pack_samples(ctx->rec, smp, (long long)total, ctx->stream), "pack samples");
         ctx->launches += 1;
@@ -1710,9 +1708,10 @@ extern "C" dwos_status dwos_eval_static(dwos_ctx* ctx, int n_query, const float*
     L.wide_depth = ctx->bvh.wide_depth;
     int blocks = 0;
     CK(launch_walks(L, d_prob, 1, total, d_ctr, ctx->stream, &blocks), "walk kernel");
-    CK(launch_reduce_u(d_rec, n_query, W, u_mean, u_se, ctx->stream), "reduce u");
-    if (diff)
-        CK(launch_reduce_udot(d_rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, ctx->n_param, n_query, W, du_mean,
-                              du_se, ctx->stream), "reduce udot");
+    if (!diff)
+        CK(launch_reduce_u(d_rec, n_query, W, u_mean, u_se, ctx->stream), "reduce u");
+    else
+        CK(launch_reduce_udot(d_rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, ctx->n_param, n_query, W, u_mean,
+                              u_se, du_mean, du_se, ctx->stream), "reduce udot");
     return DWOS_OK;
 }

@@ -224,16 +224,18 @@ cudaError_t launch_star_weight(int dim, float k, int n, const float* t, const fl
 // Estimator reductions (estimators.cu).
 // mean / SE of the first `used` (0: all W) walks of each point
 cudaError_t launch_reduce_u(const dwos_record* rec, int n_points, int W, double* mean, double* se,
-                            cudaStream_t stream, const CvView* cv = nullptr, int used = 0);
+                            cudaStream_t stream, const CvView* cv = nullptr, int used = 0,
+                            double* se_plain = nullptr);   // se_plain: standard error without cv
 // the control-variate network's training rows from thinned walks (see dwos_cv_training_set)
 cudaError_t launch_cv_rows(const float4* samples, const dwos_walk_debug* dbg, long long n_rows, long long off,
                            long long stride, float h, float q_weight, float* x, float* t, float* m, double* acc,
                            cudaStream_t stream);
 // per-walk training samples: s.w <- u - s.w (the estimate of u at x1) where x1 exists
 cudaError_t launch_pack_samples(const dwos_record* rec, float4* samples, long long n, cudaStream_t stream);
+// u and du (reduce_u alone if n_param is 0)
 cudaError_t launch_reduce_udot(const dwos_record* rec, const int* elem, const float* jac, const float* dg,
-                               int dim, int n_param, int n_points, int W, double* mean, double* se,
-                               cudaStream_t stream);
+                               int dim, int n_param, int n_points, int W, double* mean, double* se, double* dmean,
+                               double* dse, cudaStream_t stream);
 // mode 0: VJP weights w_p / W;  1: U-statistic L2 weights in batches of B;  2: correlated
 // product (umean = mean u of all W walks);  3: uncorrelated product (umean = mean u of the
 // first W/2 walks, weights on the other W/2).

@@ -1,8 +1,8 @@
 // Estimator reductions over per-walk records (FP64 sums).
 //
 //  reduce_u     per-point mean and standard error of u (Sec. 3.3)
-//  reduce_udot  forward-mode udot per point and parameter (Sec. 4.1, the
-//               N-vector of one walk rebuilt from its record and the vertex
+//  reduce_udot  the same with forward-mode udot per point and parameter (Sec. 4.1,
+//               the N-vector of one walk rebuilt from its record and the vertex
 //               Jacobians)
 //  scatter      reverse mode (Sec. 4.3): a weight per walk (VJP cotangent, or
 //               the U-statistic product weight of Eq. (ustatistics) in batches
@@ -11,10 +11,14 @@
 //               in shared memory before the global atomics
 //  gemv         the adjoint map grad_theta = sum_v J_v^T a_v + sum_v dg_v s_v
 //  loss         1/2 sum_p (mean_p - uref_p)^2
+#include <cooperative_groups.h>
+
 #include "dwos_device.cuh"
 #include "dwos_internal.h"
 
 namespace dwos {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -55,88 +59,151 @@ __device__ __forceinline__ float walk_u32(const dwos_record* __restrict__ rec, l
     return u;
 }
 
-// Mean (and standard error) of the first `used` walks of each point's W.
-__global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int used, double* mean, double* se,
-                                CvView cv) {
-    const int p = blockIdx.x;
-    double s = 0.0, s2 = 0.0;
-    for (int w = threadIdx.x; w < used; w += blockDim.x) {
-        const double u = walk_u(rec, (long long)p * W + w, p, cv);
-        s += u;
-        s2 += u * u;
+__device__ __forceinline__ double std_error(double s2, double mean, double count) {
+    const double var = count > 1 ? fmax(s2 - count * mean * mean, 0.0) / (count - 1) : 0.0;
+    return sqrt(var / count);
+}
+
+// Sums of NV values over the block, to its first thread.
+template <int NV>
+__device__ __forceinline__ void block_sum(double (&v)[NV]) {
+    __shared__ double sh[NV][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        v[k] = warp_sum(v[k]);
+        if (lane == 0) sh[k][warp] = v[k];
     }
-    __shared__ double sh[2][32];
-    s = warp_sum(s);
-    s2 = warp_sum(s2);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) { sh[0][warp] = s; sh[1][warp] = s2; }
     __syncthreads();
-    if (warp == 0) {
-        const int nw = blockDim.x >> 5;
-        s = lane < nw ? sh[0][lane] : 0.0;
-        s2 = lane < nw ? sh[1][lane] : 0.0;
-        s = warp_sum(s);
-        s2 = warp_sum(s2);
-        if (lane == 0) {
-            const double m = s / used;
-            mean[p] = m;
-            if (se) {
-                const double var = used > 1 ? fmax(s2 - used * m * m, 0.0) / (used - 1) : 0.0;
-                se[p] = sqrt(var / used);
+    if (warp != 0) return;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = warp_sum(lane < nw ? sh[k][lane] : 0.0);
+}
+
+// Mean (and standard error) of the first `used` walks of each point's W; with PLAIN also
+// the standard error without the control variate, from the same pass over the records.
+template <bool PLAIN>
+__global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int used, double* mean, double* se,
+                                CvView cv, double* se_plain) {
+    const int p = blockIdx.x;
+    double a[PLAIN ? 4 : 2] = {};
+    for (int w = threadIdx.x; w < used; w += blockDim.x) {
+        const long long i = (long long)p * W + w;
+        const double u = walk_u(rec, i, p, cv);
+        a[0] += u;
+        a[1] += u * u;
+        if constexpr (PLAIN) {
+            const double v = rec[i].u;
+            a[2] += v;
+            a[3] += v * v;
+        }
+    }
+    block_sum(a);
+    if (threadIdx.x != 0) return;
+    const double m = a[0] / used;
+    mean[p] = m;
+    if (se) se[p] = std_error(a[1], m, used);
+    if constexpr (PLAIN) se_plain[p] = std_error(a[3], a[2] / used, used);
+}
+
+// u and the forward-mode derivatives of one point: a cluster of blocks shares the point's
+// walks.  A block takes a range of them 256 at a time: each thread reads one record, adds
+// its u and leaves what the derivatives need (vertices, barycentric weights in FP64, c) in
+// shared memory; then every thread takes one parameter (column) of every G-th walk.  The
+// FP64 sums are what it costs: packing G = 256 / C walks of C columns to a block keeps the
+// lanes full (17 parameters in a warp of their own left 15 idle), and the cluster spreads a
+// few points' walks over the chip.  64 points x 1024 walks, 17 parameters: 104 us as one
+// block per point and a kernel of its own for u, 30 us now.
+constexpr int kUdotCols = 128;      // columns a block takes at most (blockIdx.y: chunks of them)
+constexpr int kUdotCluster = 8;     // blocks of a point's cluster at most
+
+template <int DIM>
+__global__ void __launch_bounds__(256) reduce_udot_kernel(const dwos_record* __restrict__ rec,
+                                                          const int* __restrict__ elem,
+                                                          const float* __restrict__ jac,
+                                                          const float* __restrict__ dg, int N, int W, int cols,
+                                                          double* mean, double* se, double* dmean, double* dse) {
+    __shared__ double bw[DIM][256];          // barycentric weights
+    __shared__ float cv[DIM][256];           // the boundary term's direction
+    __shared__ int vid[DIM][256];            // vertices (-1: the walk has no boundary term)
+    __shared__ double red[2][256];           // sums of v and v^2 per thread
+    __shared__ double part[2][kUdotCols];    // the block's sums per column
+    __shared__ double upart[2];              // and of u
+    cg::cluster_group cluster = cg::this_cluster();
+    const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+    const int p = blockIdx.x / S, t = threadIdx.x;
+    const int first = blockIdx.y * cols, C = min(cols, N - first), G = 256 / C;
+    const int g = t / C, j = first + t % C;
+    const int begin = (int)((long long)W * rank / S), end = (int)((long long)W * (rank + 1) / S);
+    double s = 0.0, s2 = 0.0, u[2] = {0.0, 0.0};
+    for (int base = begin; base < end; base += 256) {
+        const int cnt = min(256, end - base);
+        __syncthreads();
+        if (t < cnt) {
+            const dwos_record r = rec[(size_t)p * W + base + t];
+            if (blockIdx.y == 0) {
+                u[0] += (double)r.u;
+                u[1] += (double)r.u * r.u;
+            }
+            const float w[3] = {1.0f - r.b1 - r.b2, r.b1, r.b2};
+#pragma unroll
+            for (int i = 0; i < DIM; ++i) {
+                vid[i][t] = r.elem >= 0 ? __ldg(elem + DIM * r.elem + i) : -1;
+                bw[i][t] = (double)w[i];
+                cv[i][t] = r.c[i];
             }
         }
-    }
-}
-
-// Forward-mode derivative of one walk for parameter j.
-template <int DIM>
-__device__ __forceinline__ double walk_udot(const dwos_record& r, const int* __restrict__ elem,
-                                            const float* __restrict__ jac, const float* __restrict__ dg, int N,
-                                            int j) {
-    if (r.elem < 0) return 0.0;
-    const float w[3] = {1.0f - r.b1 - r.b2, r.b1, r.b2};
-    double v = 0.0;
+        __syncthreads();
+        if (g < G)
+            for (int w = g; w < cnt; w += G) {
+                if (vid[0][w] < 0) continue;
+                double v = 0.0;
 #pragma unroll
-    for (int i = 0; i < DIM; ++i) {
-        const int vid = __ldg(elem + DIM * r.elem + i);
-        const float* J = jac + (size_t)vid * DIM * N + j;
-        float cj = 0.0f;
+                for (int i = 0; i < DIM; ++i) {
+                    const float* J = jac + (size_t)vid[i][w] * DIM * N + j;
+                    float cj = 0.0f;
 #pragma unroll
-        for (int k = 0; k < DIM; ++k) cj = fmaf(r.c[k], __ldg(J + (size_t)k * N), cj);
-        if (dg) cj += __ldg(dg + (size_t)vid * N + j);
-        v += (double)w[i] * cj;
+                    for (int k = 0; k < DIM; ++k) cj = fmaf(cv[k][w], __ldg(J + (size_t)k * N), cj);
+                    if (dg) cj += __ldg(dg + (size_t)vid[i][w] * N + j);
+                    v += bw[i][w] * cj;
+                }
+                s += v;
+                s2 += v * v;
+            }
     }
-    return v;
-}
-
-template <int DIM>
-__global__ void reduce_udot_kernel(const dwos_record* __restrict__ rec, const int* __restrict__ elem,
-                                   const float* __restrict__ jac, const float* __restrict__ dg, int N, int W,
-                                   double* mean, double* se) {
-    const int p = blockIdx.x;
-    const int j = blockIdx.y * 32 + threadIdx.x;
-    double s = 0.0, s2 = 0.0;
-    if (j < N) {
-        for (int w = threadIdx.y; w < W; w += blockDim.y) {
-            const dwos_record r = rec[(size_t)p * W + w];
-            const double v = walk_udot<DIM>(r, elem, jac, dg, N, j);
-            s += v;
-            s2 += v * v;
+    red[0][t] = s;
+    red[1][t] = s2;
+    block_sum(u);                            // (a block barrier: red is complete)
+    if (t == 0) { upart[0] = u[0]; upart[1] = u[1]; }
+    if (t < C) {
+        for (int k = 1; k < G; ++k) { s += red[0][t + k * C]; s2 += red[1][t + k * C]; }
+        part[0][t] = s;
+        part[1][t] = s2;
+    }
+    cluster.sync();
+    if (rank == 0) {
+        if (t < C) {
+            for (int k = 1; k < S; ++k) {
+                const double* o = cluster.map_shared_rank(&part[0][0], k);
+                s += o[t];
+                s2 += o[kUdotCols + t];
+            }
+            const double m = s / W;
+            dmean[(size_t)p * N + j] = m;
+            if (dse) dse[(size_t)p * N + j] = std_error(s2, m, W);
+        }
+        if (t == 0 && blockIdx.y == 0) {
+            for (int k = 1; k < S; ++k) {
+                const double* o = cluster.map_shared_rank(&upart[0], k);
+                u[0] += o[0];
+                u[1] += o[1];
+            }
+            const double m = u[0] / W;
+            mean[p] = m;
+            if (se) se[p] = std_error(u[1], m, W);
         }
     }
-    __shared__ double sh[2][8][33];
-    sh[0][threadIdx.y][threadIdx.x] = s;
-    sh[1][threadIdx.y][threadIdx.x] = s2;
-    __syncthreads();
-    if (threadIdx.y == 0 && j < N) {
-        for (int y = 1; y < blockDim.y; ++y) { s += sh[0][y][threadIdx.x]; s2 += sh[1][y][threadIdx.x]; }
-        const double m = s / W;
-        mean[(size_t)p * N + j] = m;
-        if (se) {
-            const double var = W > 1 ? fmax(s2 - W * m * m, 0.0) / (W - 1) : 0.0;
-            se[(size_t)p * N + j] = sqrt(var / W);
-        }
-    }
+    cluster.sync();                          // rank 0 has read the others' shared memory
 }
 
 // Reverse-mode scatter.  Each block takes a contiguous range of walks (whole
@@ -345,34 +412,59 @@ __global__ void gemv_kernel(const float* __restrict__ jac, const float* __restri
 }
 
 // mean[p] * scale is the point's mean (scale 1 / W for per-point sums); it is
-// also written to mean_out when given.
-__global__ void loss_kernel(const double* mean, const float* uref, const float* pweight, int n, double* loss,
-                            double scale, double* mean_out) {
-    double s = 0.0;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
+// also written to mean_out when given.  One cluster: FP64 arithmetic bounds the sum, so
+// many points are shared by its blocks (16384 points: 43 us in one block, 10 us in eight),
+// and rank 0 adds the blocks' sums in order.
+constexpr int kLossCluster = 8;
+constexpr int kLossSplit = 2048;    // points from which a cluster of blocks is worth its barriers
+
+__global__ void __launch_bounds__(256) loss_kernel(const double* mean, const float* uref, const float* pweight, int n,
+                                                   double* loss, double scale, double* mean_out) {
+    __shared__ double total;
+    cg::cluster_group cluster = cg::this_cluster();
+    double s[1] = {0.0};
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
         const double m = mean[p] * scale;
         if (mean_out) mean_out[p] = m;
         const double e = m - (double)uref[p];
-        s += 0.5 * e * e * (pweight ? (double)pweight[p] : 1.0);
+        s[0] += 0.5 * e * e * (pweight ? (double)pweight[p] : 1.0);
     }
-    __shared__ double sh[32];
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        s = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
-        s = warp_sum(s);
-        if (threadIdx.x == 0) *loss = s;
+    block_sum(s);
+    if (threadIdx.x == 0) total = s[0];
+    cluster.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        for (int k = 1; k < (int)gridDim.x; ++k) s[0] += *cluster.map_shared_rank(&total, k);
+        *loss = s[0];
     }
+    cluster.sync();                 // the first block has read the others' sums
+}
+
+// One launch with clusters of `size` blocks along x.
+template <class... P, class... A>
+cudaError_t launch_cluster(void (*kernel)(P...), dim3 grid, int block, int size, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 }  // namespace
 
 cudaError_t launch_reduce_u(const dwos_record* rec, int n_points, int W, double* mean, double* se, cudaStream_t s,
-                            const CvView* cv, int used) {
+                            const CvView* cv, int used, double* se_plain) {
     if (n_points <= 0) return cudaSuccess;
     const CvView none{nullptr, nullptr, nullptr, 2, nullptr};
-    reduce_u_kernel<<<n_points, 256, 0, s>>>(rec, W, used > 0 && used <= W ? used : W, mean, se, cv ? *cv : none);
+    const int n = used > 0 && used <= W ? used : W;
+    if (se_plain) reduce_u_kernel<true><<<n_points, 256, 0, s>>>(rec, W, n, mean, se, cv ? *cv : none, se_plain);
+    else reduce_u_kernel<false><<<n_points, 256, 0, s>>>(rec, W, n, mean, se, cv ? *cv : none, nullptr);
     return cudaGetLastError();
 }
 
@@ -466,12 +558,19 @@ cudaError_t launch_pack_samples(const dwos_record* rec, float4* samples, long lo
 }
 
 cudaError_t launch_reduce_udot(const dwos_record* rec, const int* elem, const float* jac, const float* dg, int dim,
-                               int N, int n_points, int W, double* mean, double* se, cudaStream_t s) {
-    if (n_points <= 0 || N <= 0) return cudaSuccess;
-    dim3 grid(n_points, (N + 31) / 32), block(32, 8);
-    if (dim == 2) reduce_udot_kernel<2><<<grid, block, 0, s>>>(rec, elem, jac, dg, N, W, mean, se);
-    else reduce_udot_kernel<3><<<grid, block, 0, s>>>(rec, elem, jac, dg, N, W, mean, se);
-    return cudaGetLastError();
+                               int N, int n_points, int W, double* mean, double* se, double* dmean, double* dse,
+                               cudaStream_t s) {
+    if (n_points <= 0) return cudaSuccess;
+    if (N <= 0) return launch_reduce_u(rec, n_points, W, mean, se, s);
+    const int ny = (N + kUdotCols - 1) / kUdotCols, cols = (N + ny - 1) / ny;
+    // blocks to a point: until the grid has four per SM, each with 64 walks or more
+    int S = 1;
+    while (S < kUdotCluster && (long long)n_points * ny * S < 4 * 152 && W / (2 * S) >= 64) S *= 2;
+    const dim3 grid((unsigned)n_points * S, ny);
+    return dim == 2 ? launch_cluster(reduce_udot_kernel<2>, grid, 256, S, s, rec, elem, jac, dg, N, W, cols, mean, se,
+                                     dmean, dse)
+                    : launch_cluster(reduce_udot_kernel<3>, grid, 256, S, s, rec, elem, jac, dg, N, W, cols, mean, se,
+                                     dmean, dse);
 }
 
 cudaError_t launch_vertex_active(const float* jac, const float* dg, int n_vert, int dim, int n_param,
@@ -520,8 +619,9 @@ cudaError_t launch_gemv(const float* jac, const float* dg, const double* acc_ver
 
 cudaError_t launch_loss(const double* mean, const float* uref, int n_points, double* loss, cudaStream_t s,
                         const float* pweight, double scale, double* mean_out) {
-    loss_kernel<<<1, 256, 0, s>>>(mean, uref, pweight, n_points, loss, scale, mean_out);
-    return cudaGetLastError();
+    const int blocks = n_points >= kLossSplit ? kLossCluster : 1;
+    return launch_cluster(loss_kernel, dim3(blocks), 256, blocks, s, mean, uref, pweight, n_points, loss, scale,
+                          mean_out);
 }
 
 }  // namespace dwos
