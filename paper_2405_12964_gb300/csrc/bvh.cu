@@ -1,9 +1,9 @@
 // Linear BVH over boundary elements, built on the device:
 //   element boxes + scene bounds -> Morton codes -> radix sort (CUB) ->
 //   binary radix tree (Karras, "Maximizing parallelism in the construction of
-//   BVHs, octrees and k-d trees", HPG 2012) -> bottom-up box refit with
-//   arrival counters -> leaf primitives written in Morton order -> wide tree
-//   collapsed from the binary one (2D: 32 axis-aligned slots, 3D: 8 oriented ones).
+//   BVHs, octrees and k-d trees", HPG 2012) -> leaf primitives written in Morton
+//   order -> boxes over the nodes' ranges of leaves -> wide tree collapsed from the
+//   binary one (2D: 32 axis-aligned slots, 3D: 8 oriented ones).
 // Plus the batched closest-point, ray-parity inside test and Philox kernels.
 #include <cub/device/device_radix_sort.cuh>
 
@@ -259,47 +259,71 @@ __device__ __forceinline__ void write_child_box(float4* nodes, int node, int slo
     }
 }
 
+// ---- boxes ----------------------------------------------------------------
+// A node's box is the union over its contiguous range of leaves.  Climbing from every
+// leaf with an arrival counter per node, a fence and an atomic per level, the boxes of
+// 4,100 segments took 35 us, all of it the chain of a dozen dependent levels.  Instead
+// one launch writes the leaves and the boxes of their aligned blocks of 8, 64 and 512,
+// and a second covers each node's range by at most seven leaves or blocks on each side
+// per level, all loaded independently: 9 us.
+constexpr int kLeafBlock = 512;      // leaves of a block, and of the highest level's boxes
+
+// Box k of level 1..3 (8, 64, 512 leaves) among nt leaves.
 template <int DIM>
-__global__ void refit_kernel(const float* vert, const int* elem, const int* sorted_elem, int n,
-                             const int* node_child, const int* node_parent, const int* leaf_parent,
-                             int* counters, float4* nodes) {
-    const int leaf = blockIdx.x * blockDim.x + threadIdx.x;
-    if (leaf >= n) return;
-    float lo[DIM], hi[DIM];
-    elem_box<DIM>(vert, elem, sorted_elem[leaf], lo, hi);
-    int child = ~leaf;
-    int node = leaf_parent[leaf];
-    while (node >= 0) {
-        const int slot = (node_child[2 * node] == child) ? 0 : 1;
-        write_child_box<DIM>(nodes, node, slot, lo, hi);
-        __threadfence();                                   // publish this child's box
-        if (atomicAdd(counters + node, 1) == 0) return;    // the sibling finishes this node
-        __threadfence();
-        // second arrival: the node's bounds are the union of both child slots (read through L2)
-        const volatile float* f = reinterpret_cast<const volatile float*>(nodes + BvhLayout<DIM>::kNodeF4 * node);
+__device__ __forceinline__ float4* level_box(float4* boxes, int nt, int level, int k) {
+    const int n8 = (nt + 7) / 8, n64 = (nt + 63) / 64;
+    return boxes + (DIM == 2 ? 1 : 2) * ((level > 1 ? n8 : 0) + (level > 2 ? n64 : 0) + (size_t)k);
+}
+__host__ inline size_t level_boxes(size_t n) { return (n + 7) / 8 + (n + 63) / 64 + (n + 511) / 512; }
+
+template <int DIM>
+__device__ __forceinline__ void store_level_box(float4* b, const float* lo, const float* hi) {
+    if (DIM == 2) {
+        *b = make_float4(lo[0], lo[1], hi[0], hi[1]);
+    } else {
+        b[0] = make_float4(lo[0], lo[1], lo[DIM - 1], 0.0f);
+        b[1] = make_float4(hi[0], hi[1], hi[DIM - 1], 0.0f);
+    }
+}
+template <int DIM>
+__device__ __forceinline__ void add_level_box(const float4* b, float* lo, float* hi) {
+    const float4 p = __ldg(b);
+    const float4 q = DIM == 2 ? make_float4(p.z, p.w, 0.0f, 0.0f) : __ldg(b + 1);
+    lo[0] = fminf(lo[0], p.x); lo[1] = fminf(lo[1], p.y);
+    hi[0] = fmaxf(hi[0], q.x); hi[1] = fmaxf(hi[1], q.y);
+    if (DIM == 3) { lo[DIM - 1] = fminf(lo[DIM - 1], p.z); hi[DIM - 1] = fmaxf(hi[DIM - 1], q.z); }
+}
+
+// Union over groups of eight lanes.
+template <int DIM>
+__device__ __forceinline__ void union8(unsigned mask, float* lo, float* hi) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) {
 #pragma unroll
         for (int k = 0; k < DIM; ++k) {
-            float a_lo, a_hi, b_lo, b_hi;
-            if (DIM == 2) { a_lo = f[k]; a_hi = f[2 + k]; b_lo = f[4 + k]; b_hi = f[6 + k]; }
-            else { a_lo = f[k]; a_hi = f[3 + k]; b_lo = f[6 + k]; b_hi = f[9 + k]; }
-            lo[k] = fminf(a_lo, b_lo);
-            hi[k] = fmaxf(a_hi, b_hi);
+            lo[k] = fminf(lo[k], __shfl_xor_sync(mask, lo[k], o));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(mask, hi[k], o));
         }
-        child = node;
-        node = node_parent[node];
     }
 }
 
+// The leaves (vertices, elements), the nodes' links and, over the nt >= 2 leaves of a
+// tree, the leaves' own boxes in their parents and the level boxes.
 template <int DIM>
-__global__ void finalize_kernel(const float* vert, const int* elem, const int* sorted_elem, int n,
-                                const int* node_child, const int* node_parent, int n_internal,
-                                float4* nodes, float4* prims, int* prim_elem, int* leaf_of_elem) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_internal && node_child) {
+__global__ void __launch_bounds__(kLeafBlock)
+    leaves_kernel(const float* vert, const int* elem, const int* sorted_elem, int n, int nt, const int* node_child,
+                  const int* node_parent, const int* leaf_parent, float4* nodes, float4* prims, int* prim_elem,
+                  int* leaf_of_elem, float4* boxes) {
+    const int i = blockIdx.x * kLeafBlock + threadIdx.x, t = threadIdx.x;
+    const bool tree = nt >= 2;
+    if (tree && i < nt - 1) {
         float4* m = nodes + BvhLayout<DIM>::kNodeF4 * i + (BvhLayout<DIM>::kNodeF4 - 1);
         *m = make_float4(__int_as_float(node_child[2 * i]), __int_as_float(node_child[2 * i + 1]),
                          __int_as_float(node_parent[i]), 0.0f);
     }
+    float lo[DIM], hi[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) { lo[k] = kInf; hi[k] = -kInf; }
     if (i < n) {
         const int e = sorted_elem[i];
         prim_elem[i] = e;
@@ -314,6 +338,79 @@ __global__ void finalize_kernel(const float* vert, const int* elem, const int* s
                 prims[3 * i + c] = make_float4(vert[3 * v], vert[3 * v + 1], vert[3 * v + 2], 0.0f);
             }
         }
+        if (tree && i < nt) {
+            elem_box<DIM>(vert, elem, e, lo, hi);
+            const int parent = leaf_parent[i];
+            write_child_box<DIM>(nodes, parent, node_child[2 * parent] == ~i ? 0 : 1, lo, hi);
+        }
+    }
+    if (!tree || blockIdx.x * kLeafBlock >= nt) return;      // whole blocks
+    __shared__ float sb[kLeafBlock / 8][2 * DIM];
+    union8<DIM>(0xffffffffu, lo, hi);
+    auto put = [&](int level, int k, int slot) {
+        if (k * (level == 1 ? 8 : level == 2 ? 64 : 512) < nt) store_level_box<DIM>(level_box<DIM>(boxes, nt, level, k), lo, hi);
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) { sb[slot][j] = lo[j]; sb[slot][DIM + j] = hi[j]; }
+    };
+    auto get = [&](int slot) {
+#pragma unroll
+        for (int j = 0; j < DIM; ++j) { lo[j] = sb[slot][j]; hi[j] = sb[slot][DIM + j]; }
+    };
+    if (t % 8 == 0) put(1, i / 8, t / 8);
+    __syncthreads();
+    if (t < 64) {
+        get(t);
+        union8<DIM>(0xffffffffu, lo, hi);
+    }
+    __syncthreads();
+    if (t < 64 && t % 8 == 0) put(2, blockIdx.x * 8 + t / 8, t / 8);
+    __syncthreads();
+    if (t < 8) {
+        get(t);
+        union8<DIM>(0xffu, lo, hi);
+        if (t == 0) store_level_box<DIM>(level_box<DIM>(boxes, nt, 3, blockIdx.x), lo, hi);
+    }
+}
+
+// The inner nodes' boxes in their parents: eight lanes to a node.
+template <int DIM>
+__global__ void node_boxes_kernel(const float4* prims, float4* boxes, int nt, const int* node_child,
+                                  const int* node_parent, const int* node_count, const int* node_first,
+                                  float4* nodes) {
+    const int c = (blockIdx.x * blockDim.x + threadIdx.x) / 8 + 1, j = threadIdx.x % 8;   // the root has no parent
+    float lo[DIM], hi[DIM];
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) { lo[k] = kInf; hi[k] = -kInf; }
+    if (c < nt - 1) {
+        int a = node_first[c], b = a + node_count[c];
+        auto add = [&](int level, int k) {
+            if (level == 0) {
+                float l[DIM], h[DIM];
+                prim_box<DIM>(prims, k, l, h);
+#pragma unroll
+                for (int q = 0; q < DIM; ++q) { lo[q] = fminf(lo[q], l[q]); hi[q] = fmaxf(hi[q], h[q]); }
+            } else {
+                add_level_box<DIM>(level_box<DIM>(boxes, nt, level, k), lo, hi);
+            }
+        };
+#pragma unroll
+        for (int level = 0; level < 4; ++level) {
+            const int na = (a + 7) >> 3, nb = b >> 3;
+            if (level == 3 || na >= nb) {
+                for (int k = a + j; k < b; k += 8) add(level, k);
+                break;
+            }
+            if (a + j < 8 * na) add(level, a + j);
+            if (8 * nb + j < b) add(level, 8 * nb + j);
+            a = na;
+            b = nb;
+        }
+    }
+    __syncwarp();
+    union8<DIM>(0xffffffffu, lo, hi);
+    if (c < nt - 1 && j == 0) {
+        const int parent = node_parent[c];
+        write_child_box<DIM>(nodes, parent, node_child[2 * parent] == c ? 0 : 1, lo, hi);
     }
 }
 
@@ -788,15 +885,18 @@ __device__ __forceinline__ void project(const RayFrame& F, const float* o, float
     z = __fadd_rn(__fadd_rn(__fmul_rn(dx, F.dir[0]), __fmul_rn(dy, F.dir[1])), __fmul_rn(dz, F.dir[2]));
 }
 
+__device__ __forceinline__ float ray_segment_t(float4 s, const float* o, const float* dir) {
+    const float sa = side2(o, dir, s.x, s.y), sb = side2(o, dir, s.z, s.w);
+    if ((sa >= 0.0f) == (sb >= 0.0f)) return -1.0f;
+    const float lam = sa / (sa - sb);
+    const float ax = s.x - o[0], ay = s.y - o[1];
+    return (ax + lam * (s.z - s.x)) * dir[0] + (ay + lam * (s.w - s.y)) * dir[1];
+}
+
 template <int DIM>
 __device__ __forceinline__ float ray_prim_t(const float4* prims, int p, const float* o, const RayFrame& F) {
     if (DIM == 2) {
-        const float4 s = prims[p];
-        const float sa = side2(o, F.dir, s.x, s.y), sb = side2(o, F.dir, s.z, s.w);
-        if ((sa >= 0.0f) == (sb >= 0.0f)) return -1.0f;
-        const float lam = sa / (sa - sb);
-        const float ax = s.x - o[0], ay = s.y - o[1];
-        return (ax + lam * (s.z - s.x)) * F.dir[0] + (ay + lam * (s.w - s.y)) * F.dir[1];
+        return ray_segment_t(prims[p], o, F.dir);
     } else {
         float ax, ay, az, bx, by, bz, cx, cy, cz;
         project(F, o, prims[3 * p], ax, ay, az);
@@ -811,20 +911,6 @@ __device__ __forceinline__ float ray_prim_t(const float4* prims, int p, const fl
         const float den = wa + wb + wc;
         if (den == 0.0f) return -1.0f;
         return (wa * az + wb * bz + wc * cz) / den;
-    }
-}
-
-template <int DIM>
-__device__ __forceinline__ void prim_box(const float4* prims, int p, float* lo, float* hi) {
-    if (DIM == 2) {
-        const float4 s = prims[p];
-        lo[0] = fminf(s.x, s.z); hi[0] = fmaxf(s.x, s.z);
-        lo[1] = fminf(s.y, s.w); hi[1] = fmaxf(s.y, s.w);
-    } else {
-        const float4 a = prims[3 * p], b = prims[3 * p + 1], c = prims[3 * p + 2];
-        lo[0] = fminf(a.x, fminf(b.x, c.x)); hi[0] = fmaxf(a.x, fmaxf(b.x, c.x));
-        lo[1] = fminf(a.y, fminf(b.y, c.y)); hi[1] = fmaxf(a.y, fmaxf(b.y, c.y));
-        lo[2] = fminf(a.z, fminf(b.z, c.z)); hi[2] = fmaxf(a.z, fmaxf(b.z, c.z));
     }
 }
 
@@ -887,30 +973,32 @@ __global__ void inside_kernel(BvhView bvh, int n, const float* p, int* inside, c
         count += (t > 0.0f && t >= ta && t < tb) ? 1 : 0;
     }
     if (bvh.n_internal > 0) {
-        int node = bvh.root, from = kFromParent;
-        int budget = 3 * bvh.n_internal + 8;
+        int st[kLaneStack], sp = 0, node = bvh.root;
+        int budget = bvh.n_internal + 8;
         while (--budget >= 0) {
             float lo0[DIM], hi0[DIM], lo1[DIM], hi1[DIM];
             int c0, c1, parent;
             load_node<DIM>(bvh.nodes, node, lo0, hi0, lo1, hi1, c0, c1, parent);
-            int state = from == kFromParent ? 0 : (from == c0 ? 1 : 2);
-            int next = kFromParent;
-            while (state < 2) {
-                const int c = state == 0 ? c0 : c1;
-                const bool hit = c != kEmptyChild &&
-                                 (state == 0 ? seg_hits_box<DIM>(o, inv, ta, tb, lo0, hi0)
-                                             : seg_hits_box<DIM>(o, inv, ta, tb, lo1, hi1));
-                if (hit && c >= 0) { next = c; break; }
-                if (hit) {
+            int next = kNoNode;
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                const int c = side == 0 ? c0 : c1;
+                if (c == kEmptyChild || !(side == 0 ? seg_hits_box<DIM>(o, inv, ta, tb, lo0, hi0)
+                                                    : seg_hits_box<DIM>(o, inv, ta, tb, lo1, hi1))) continue;
+                if (c < 0) {
                     const float t = ray_prim_t<DIM>(bvh.prims, ~c, o, F);
                     count += (t > 0.0f && t >= ta && t < tb) ? 1 : 0;
+                } else if (next == kNoNode) {
+                    next = c;
+                } else if (sp < kLaneStack) {     // (a path has at most 62 nodes)
+                    st[sp++] = c;
                 }
-                ++state;
             }
-            if (next != kFromParent) { from = kFromParent; node = next; continue; }
-            if (parent < 0) break;
-            from = node;
-            node = parent;
+            if (next == kNoNode) {
+                if (sp == 0) break;
+                next = st[--sp];
+            }
+            node = next;
         }
     }
     for (int off = 16; off > 0; off >>= 1) count += __shfl_xor_sync(0xffffffffu, count, off);
@@ -965,7 +1053,7 @@ cudaError_t bvh_reserve(BvhBuffers& b, int dim, int n_elem) {
     DW_TRY(cudaMalloc(&b.leaf_parent, sizeof(int) * (size_t)n_elem));
     DW_TRY(cudaMalloc(&b.node_parent, sizeof(int) * (size_t)n_int));
     DW_TRY(cudaMalloc(&b.node_child, sizeof(int) * 2 * (size_t)n_int));
-    DW_TRY(cudaMalloc(&b.counters, sizeof(int) * (size_t)n_int));
+    DW_TRY(cudaMalloc(&b.boxes, sizeof(float4) * (dim == 2 ? 1 : 2) * level_boxes((size_t)n_elem)));
     DW_TRY(cudaMalloc(&b.node_count, sizeof(int) * 2 * (size_t)n_int));   // leaf counts, then first leaves
     DW_TRY(cudaMalloc(&b.node_cell, sizeof(float) * 2 * dim * (size_t)n_int));
     DW_TRY(cudaMalloc(&b.wroot, sizeof(int) * 2 * (size_t)n_int));        // roots, then first inner children
@@ -985,13 +1073,26 @@ cudaError_t bvh_reserve(BvhBuffers& b, int dim, int n_elem) {
 void bvh_free(BvhBuffers& b) {
     cudaFree(b.nodes); cudaFree(b.prims); cudaFree(b.prim_elem); cudaFree(b.leaf_of_elem); cudaFree(b.keys); cudaFree(b.keys_sorted);
     cudaFree(b.vals); cudaFree(b.vals_sorted); cudaFree(b.leaf_parent); cudaFree(b.node_parent);
-    cudaFree(b.node_child); cudaFree(b.counters); cudaFree(b.bounds); cudaFree(b.stats); cudaFree(b.node_cell);
+    cudaFree(b.node_child); cudaFree(b.boxes); cudaFree(b.bounds); cudaFree(b.stats); cudaFree(b.node_cell);
     cudaFree(b.sort_tmp);
     cudaFree(b.wnodes); cudaFree(b.wsrc); cudaFree(b.wroot); cudaFree(b.wlev); cudaFree(b.node_count);
     b = BvhBuffers();
 }
 
 constexpr int kMaxBig = 64;
+
+// Leaves, links and, for a tree of two leaves or more, all boxes of the binary tree.
+template <int DIM>
+static void fill_boxes(BvhBuffers& b, const float* vert, const int* elem, cudaStream_t s) {
+    const int nt = b.n_tree;
+    leaves_kernel<DIM><<<nblk(b.n_elem, kLeafBlock), kLeafBlock, 0, s>>>(
+        vert, elem, b.vals_sorted, b.n_elem, nt, b.node_child, b.node_parent, b.leaf_parent, b.nodes, b.prims,
+        b.prim_elem, b.leaf_of_elem, b.boxes);
+    if (nt >= 3)
+        node_boxes_kernel<DIM><<<nblk(8LL * (nt - 2), 256), 256, 0, s>>>(b.prims, b.boxes, nt, b.node_child,
+                                                                         b.node_parent, b.node_count,
+                                                                         b.node_count + (nt - 1), b.nodes);
+}
 
 // The wide tree's boxes (and, in 2D, leaf children's vertices) from the binary tree.
 template <int DIM>
@@ -1095,13 +1196,7 @@ static cudaError_t build_impl(BvhBuffers& b, const float* vert, const int* elem,
         radix_tree_kernel<DIM><<<nblk(nt - 1, 256), 256, 0, s>>>(b.keys_sorted, nt, b.node_child, b.node_parent,
                                                                  b.leaf_parent, b.bounds, b.node_cell,
                                                                  b.node_count, b.node_count + (nt - 1));
-        e = cudaMemsetAsync(b.counters, 0, sizeof(int) * (size_t)(nt - 1), s);
-        if (e != cudaSuccess) return e;
-        refit_kernel<DIM><<<nblk(nt, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, nt, b.node_child,
-                                                        b.node_parent, b.leaf_parent, b.counters, b.nodes);
-        finalize_kernel<DIM><<<nblk(n, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, n, b.node_child,
-                                                          b.node_parent, nt - 1, b.nodes, b.prims, b.prim_elem,
-                                                          b.leaf_of_elem);
+        fill_boxes<DIM>(b, vert, elem, s);
         e = build_wide<DIM>(b, s);
         if (e != cudaSuccess) return e;
     } else {
@@ -1111,8 +1206,7 @@ static cudaError_t build_impl(BvhBuffers& b, const float* vert, const int* elem,
         b.n_internal = nt;    // 1: a single-leaf node; 0: no tree
         if (nt == 1) single_leaf_kernel<DIM><<<1, 1, 0, s>>>(vert, elem, b.vals_sorted, b.nodes, b.leaf_parent,
                                                              b.node_cell);
-        finalize_kernel<DIM><<<nblk(n, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, n, nullptr, nullptr, 0,
-                                                          b.nodes, b.prims, b.prim_elem, b.leaf_of_elem);
+        fill_boxes<DIM>(b, vert, elem, s);
     }
     return cudaGetLastError();
 }
@@ -1131,22 +1225,15 @@ static cudaError_t refit_impl(BvhBuffers& b, const float* vert, const int* elem,
     const int n = b.n_elem, nt = b.n_tree;
     if (n <= 0) return cudaSuccess;
     if (nt >= 2) {
-        cudaError_t e = cudaMemsetAsync(b.counters, 0, sizeof(int) * (size_t)(nt - 1), s);
-        if (e != cudaSuccess) return e;
-        refit_kernel<DIM><<<nblk(nt, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, nt, b.node_child,
-                                                        b.node_parent, b.leaf_parent, b.counters, b.nodes);
-        finalize_kernel<DIM><<<nblk(n, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, n, b.node_child,
-                                                          b.node_parent, nt - 1, b.nodes, b.prims, b.prim_elem,
-                                                          b.leaf_of_elem);
+        fill_boxes<DIM>(b, vert, elem, s);
         if (b.n_wide > 0) {
-            e = fill_wide<DIM>(b, s);
+            const cudaError_t e = fill_wide<DIM>(b, s);
             if (e != cudaSuccess) return e;
         }
     } else {
         if (nt == 1) single_leaf_kernel<DIM><<<1, 1, 0, s>>>(vert, elem, b.vals_sorted, b.nodes, b.leaf_parent,
                                                              b.node_cell);
-        finalize_kernel<DIM><<<nblk(n, 256), 256, 0, s>>>(vert, elem, b.vals_sorted, n, nullptr, nullptr, 0,
-                                                          b.nodes, b.prims, b.prim_elem, b.leaf_of_elem);
+        fill_boxes<DIM>(b, vert, elem, s);
     }
     b.cells_ok = false;
     return cudaGetLastError();

@@ -13,7 +13,6 @@
 
 namespace dwos {
 
-constexpr int kFromParent = 0x7fffffff;   // inside test's traversal: entered from above
 constexpr int kEmptyChild = 0x7ffffffe;   // child slot with an empty box
 constexpr float kInf = __builtin_inff();
 
@@ -308,10 +307,9 @@ __device__ __forceinline__ float prim_dist2(const float4* __restrict__ prims, in
     }
 }
 
-// Squared distance from q to the bounding box of leaf p.
+// Bounding box of leaf p.
 template <int DIM>
-__device__ __forceinline__ float prim_box_dist2(const float4* __restrict__ prims, int p, const float* q) {
-    float lo[DIM], hi[DIM];
+__device__ __forceinline__ void prim_box(const float4* __restrict__ prims, int p, float* lo, float* hi) {
     if (DIM == 2) {
         const float4 s = __ldg(prims + p);
         lo[0] = fminf(s.x, s.z); hi[0] = fmaxf(s.x, s.z);
@@ -322,6 +320,13 @@ __device__ __forceinline__ float prim_box_dist2(const float4* __restrict__ prims
         lo[1] = fminf(a.y, fminf(b.y, c.y)); hi[1] = fmaxf(a.y, fmaxf(b.y, c.y));
         lo[DIM - 1] = fminf(a.z, fminf(b.z, c.z)); hi[DIM - 1] = fmaxf(a.z, fmaxf(b.z, c.z));
     }
+}
+
+// Squared distance from q to the bounding box of leaf p.
+template <int DIM>
+__device__ __forceinline__ float prim_box_dist2(const float4* __restrict__ prims, int p, const float* q) {
+    float lo[DIM], hi[DIM];
+    prim_box<DIM>(prims, p, lo, hi);
     return box_dist2<DIM>(q, lo, hi);
 }
 

@@ -140,7 +140,7 @@ struct BvhBuffers {
     int* leaf_parent = nullptr;
     int* node_parent = nullptr;
     int* node_child = nullptr;    // 2 per internal node
-    int* counters = nullptr;
+    float4* boxes = nullptr;         // of aligned blocks of 8, 64 and 512 leaves
     int* node_count = nullptr;       // per internal node: leaves under it; then (second half) its first leaf
     float* node_cell = nullptr;      // Morton cell box per internal node
     float r_max = 0.0f;              // largest element half box diagonal (tree elements)
