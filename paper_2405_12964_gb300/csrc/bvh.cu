@@ -1011,6 +1011,52 @@ __global__ void inside_kernel(BvhView bvh, int n, const float* p, int* inside, c
     }
 }
 
+// The same for segments with a wide tree: a warp per point, one child of the current
+// node per lane, in any order (every leaf that the ray's line can cross is counted once).
+// Bound by the chain of node fetches, three levels of them for 4096 segments instead of
+// a dozen (256 points: 29 us by intervals of the ray on the binary tree).
+constexpr int kInsideBlock = 128;
+
+__global__ void __launch_bounds__(kInsideBlock) inside_wide_kernel(const float* wnodes, const float4* prims, int n_tree,
+                                                                   int n_big, int n, const float* p, int* inside,
+                                                                   const float* prev, float* prev_out) {
+    __shared__ int stacks[kInsideBlock / 32][kWideStack];
+    const int pt = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    int* stk = stacks[threadIdx.x >> 5];
+    if (pt >= n) return;    // whole warps exit together
+    const float dir[2] = {0.8191520443f, 0.5735764364f};
+    const float o[2] = {p[2 * pt], p[2 * pt + 1]}, inv[2] = {1.0f / dir[0], 1.0f / dir[1]};
+    if (prev && __float_as_uint(o[0]) == __float_as_uint(prev[2 * pt]) &&
+        __float_as_uint(o[1]) == __float_as_uint(prev[2 * pt + 1])) return;   // the same point as last time: its flag stands
+    int count = 0;
+    for (int q = n_tree + lane; q < n_tree + n_big; q += 32) count += ray_segment_t(prims[q], o, dir) > 0.0f ? 1 : 0;
+    int top = 0, cur = 0;
+    for (;;) {
+        const float* f = wnodes + (size_t)cur * kWideFloats;
+        const float4 s = __ldg(reinterpret_cast<const float4*>(f) + lane);
+        const int code = __float_as_int(__ldg(f + 4 * kWide + lane));
+        if (code < 0) count += ray_segment_t(s, o, dir) > 0.0f ? 1 : 0;
+        const float lo[2] = {s.x, s.y}, hi[2] = {s.z, s.w};
+        const bool hit = code >= 0 && code != kEmptyChild && seg_hits_box<2>(o, inv, 0.0f, kInf, lo, hi);
+        const unsigned m = __ballot_sync(0xffffffffu, hit);
+        __syncwarp();
+        if (hit) {
+            const int at = top + __popc(m & ((1u << lane) - 1u));
+            if (at < kWideStack) stk[at] = code;       // (31 x the depth + 1 entries at most)
+        }
+        top = min(top + __popc(m), kWideStack);
+        __syncwarp();
+        if (top == 0) break;
+        cur = stk[--top];
+    }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if (lane == 0) {
+        inside[pt] = count & 1;
+        if (prev_out) { prev_out[2 * pt] = o[0]; prev_out[2 * pt + 1] = o[1]; }
+    }
+}
+
 __global__ void philox_kernel(int n, const uint32_t* ctr, uint32_t k0, uint32_t k1, uint32_t* out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -1279,7 +1325,10 @@ cudaError_t launch_closest(const BvhBuffers& b, int n, const float* p, const int
 cudaError_t launch_inside(const BvhBuffers& b, int n, const float* p, int* inside, cudaStream_t s,
                           const float* prev, float* prev_out) {
     if (n <= 0) return cudaSuccess;
-    if (b.dim == 2) inside_kernel<2><<<nblk(32LL * n, 128), 128, 0, s>>>(view_of(b), n, p, inside, prev, prev_out);
+    if (b.dim == 2 && b.wide_ok && b.n_wide > 0)
+        inside_wide_kernel<<<nblk(32LL * n, kInsideBlock), kInsideBlock, 0, s>>>(b.wnodes, b.prims, b.n_tree, b.n_big, n, p,
+                                                                                 inside, prev, prev_out);
+    else if (b.dim == 2) inside_kernel<2><<<nblk(32LL * n, 128), 128, 0, s>>>(view_of(b), n, p, inside, prev, prev_out);
     else inside_kernel<3><<<nblk(32LL * n, 128), 128, 0, s>>>(view_of(b), n, p, inside, prev, prev_out);
     return cudaGetLastError();
 }

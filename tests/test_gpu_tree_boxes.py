@@ -68,3 +68,25 @@ def _check(rng, v, e, jac):
             want = _distances(p.astype(np.float64), np.asarray(s.current_vertices(), np.float64), e)
             # FP32 differences of coordinates of size 2: a few units of 2^-23 absolute
             assert np.abs(got.double().cpu().numpy() - want).max() <= 16 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("size", [3, 31, 32, 33, 64, 65, 1025, 4097, 40000])
+def test_inside(size):
+    rng = np.random.default_rng(size)
+    ang = np.arange(size) * 2 * np.pi / size
+    v = (1 + 0.3 * np.cos(5 * ang))[:, None] * np.stack([np.cos(ang), np.sin(ang)], 1)
+    v = v.astype(np.float32)
+    e = np.stack([np.arange(size), (np.arange(size) + 1) % size], 1).astype(np.int32)
+    p = rng.uniform(-1.5, 1.5, size=(300, 2)).astype(np.float32)
+    s = dwos.Solver(0)
+    s.set_boundary(v, e)
+    got = s.inside(p).cpu().numpy()
+    v, p = v.astype(np.float64), p.astype(np.float64)
+    a, b = v, np.roll(v, -1, 0)
+    want = np.zeros(len(p), int)
+    for i, x in enumerate(p):      # crossings of the ray towards +x
+        up = (a[:, 1] > x[1]) != (b[:, 1] > x[1])
+        cross = a[up, 0] + (x[1] - a[up, 1]) * (b[up, 0] - a[up, 0]) / (b[up, 1] - a[up, 1])
+        want[i] = (cross > x[0]).sum() & 1
+    clear = _distances(p, v, e) > 1e-5       # away from the boundary both are exact
+    assert (got[clear] == want[clear]).all()
