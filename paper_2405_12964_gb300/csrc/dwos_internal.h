@@ -195,6 +195,7 @@ struct WalkLaunch {
     bool star = false;          // walk on stars (one problem with a Neumann part)
     bool cones = false;         // walk on stars whose silhouette tree has normal cones
     bool data = false;          // walk on stars with Neumann data (runs without the cones)
+    bool few = false;           // few walks per SM (set by launch_walks)
 };
 // The problems come from the device table d_probs, or (one problem, d_probs
 // NULL) by value from host_prob.  zero_counters, when given, is zeroed by the

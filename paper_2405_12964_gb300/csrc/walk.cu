@@ -127,8 +127,13 @@ __device__ __forceinline__ void sphere_dir(const U4& r, float* om) {
 // launch; the Dirichlet part's distance queries take the launch's search
 // order, the Neumann queries per lane).  DATA: the Neumann part carries data
 // du/dn (a separate instantiation, so that reflecting walks keep their code).
-template <int DIM, bool WIDE, bool STAR = false, bool CONES = false, bool DATA = false>
-__global__ void __launch_bounds__(256, STAR ? 3 : ((DIM == 2 || WIDE) ? 4 : 3))
+// FEW: a launch of few walks over triangles, whose time is the latency of its longest
+// walks: three blocks per SM and 80 registers instead of four and 64 (166,500 walks over
+// 10,600 triangles 2.30 -> 2.11 ms, 333,000 3.16 -> 2.91; even at 666,000; above, more
+// warps hide more: 4.2 M walks over 200k triangles 48.4 against 50.5 ms).  With Neumann
+// data on segments four blocks (three: 6.5 against 6.05 ms on the thermal slab).
+template <int DIM, bool WIDE, bool STAR = false, bool CONES = false, bool DATA = false, bool FEW = false>
+__global__ void __launch_bounds__(256, STAR ? (DIM == 2 && DATA ? 4 : 3) : DIM == 2 || (WIDE && !FEW) ? 4 : 3)
     walk_kernel(const DevProblem* __restrict__ g_probs, int n_probs, unsigned long long total,
                 DevCounters* __restrict__ ctr, DevCounters* __restrict__ zero_ctr, int stk_cap,
                 int lanes, const __grid_constant__ DevProblem p_arg) {
@@ -793,6 +798,8 @@ cudaError_t launch_neumann_orient(int n, const int* behind_inside, float4* q_sta
 
 namespace {
 
+constexpr unsigned long long kFewWalks = 4096;   // walks per SM below which a launch is FEW (four lanes' worth)
+
 bool wide_launch(const WalkLaunch& L) { return L.traversal == 2 || L.traversal == 3; }
 
 int stack_entries(const WalkLaunch& L) { return wide_launch(L) ? wide_stack_entries(L.dim, L.wide_depth) : 0; }
@@ -813,6 +820,7 @@ cudaError_t with_kernel(const WalkLaunch& L, F f) {
         if (wide) return L.dim == 2 ? f(walk_kernel<2, true, true>) : f(walk_kernel<3, true, true>);
         return L.dim == 2 ? f(walk_kernel<2, false, true>) : f(walk_kernel<3, false, true>);
     }
+    if (wide && L.dim == 3 && L.few) return f(walk_kernel<3, true, false, false, false, true>);
     if (wide) return L.dim == 2 ? f(walk_kernel<2, true>) : f(walk_kernel<3, true>);
     return L.dim == 2 ? f(walk_kernel<2, false>) : f(walk_kernel<3, false>);
 }
@@ -832,7 +840,7 @@ int walk_max_blocks_per_sm(const WalkLaunch& L) {
     return n;
 }
 
-cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_probs, unsigned long long total,
+cudaError_t launch_walks(const WalkLaunch& launch, const DevProblem* d_probs, int n_probs, unsigned long long total,
                          DevCounters* d_counters, cudaStream_t stream, int* blocks_used, const DevProblem* host_prob,
                          DevCounters* zero_counters) {
     if (n_probs < 1 || n_probs > kMaxProblems) return cudaErrorInvalidValue;
@@ -842,6 +850,8 @@ cudaError_t launch_walks(const WalkLaunch& L, const DevProblem* d_probs, int n_p
         if (zero_counters) return cudaMemsetAsync(zero_counters, 0, sizeof(DevCounters), stream);
         return cudaSuccess;
     }
+    WalkLaunch L = launch;
+    L.few = total < kFewWalks * L.n_sm;
     const int bs = L.block_size;
     if (bs % 32 != 0) return cudaErrorInvalidValue;
     if (L.star && n_probs != 1) return cudaErrorInvalidValue;
