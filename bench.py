@@ -682,7 +682,7 @@ def main():
     ap.add_argument("--no-extras", action="store_true",
                     help="skip the C3 / C4 / C5 summaries that the default line carries after the C2 figures")
     ap.add_argument("--traversal", type=int, default=-1,
-                    help="closest-point search: 0 binary per lane, 1 climb, 2 32-wide warp-wide, 3 routed "
+                    help="closest-point search: 0 binary per lane, 1 climb, 2 wide tree warp-wide, 3 routed "
                          "(only queries that reach inside the binary root's child boxes are searched, warp-wide; "
                          "-1: 3)")
     args = ap.parse_args()
@@ -792,12 +792,13 @@ def main():
     rel = rmse / float(np.sqrt(np.mean(g_ref ** 2)))
 
     # roofline of the walk kernel: algorithmic bytes = binary node fetches x 48 / 64 B
-    # + 32-wide node visits x (2 dim + 1 + dim^2) x 128 B (leaf vertices included)
+    # + wide-node visits in units of 32 child slots x 640 B (2D: a float4 and a code per
+    # slot, leaf segments included) / 2048 B (3D: four nodes of 8 oriented boxes)
     # + element fetches outside the nodes (the previous step's element, outsized
     # elements; all element tests of the binary search) x 16 / 48 B
     # + one 32 B record per walk + 8 B query load per walk
     node_b = 48 if sc.dim == 2 else 64
-    wide_b = (2 * sc.dim + 1 + sc.dim * sc.dim) * 128
+    wide_b = 640 if sc.dim == 2 else 2048
     prim_b = 16 if sc.dim == 2 else 48
     alg_bytes = nodes * node_b + wnodes * wide_b + prims * prim_b + args.steps * total * (32 + 8)
     walk_s = sum(kernel_ms) / 1e3
@@ -848,8 +849,8 @@ def main():
             "config": {"workload": WORKLOADS[args.workload], "points": n_pts, "walks_per_point": W, "K": sc.K, "B": sc.B,
                        "n_param": sc.n_param, "eps": sc.eps, "h": sc.h,
                        "closest_point_search": {0: "binary LBVH, per lane", 1: "binary LBVH climbing from the hint",
-                                                2: "32-wide BVH, warp-wide",
-                                                3: "routed: binary-root test per query, then the 32-wide BVH "
+                                                2: "wide BVH (2D 32, 3D 8 children), warp-wide",
+                                                3: "routed: binary-root test per query, then the wide BVH "
                                                    "warp-wide for the queries that need the tree"}[trav],
                        "l2": "flushed between timed steps (256 MB write outside the events)",
                        "timing": ("timed steps enqueued back to back, each between its own CUDA events; "

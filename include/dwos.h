@@ -87,16 +87,18 @@ typedef struct {
     int traversal;      /* distance-query search order: 0 = binary tree from the root,
                            one query per lane, bounded by the previous step's
                            element; 1 = climbing from that element's leaf with
-                           the Morton-cell stop test; 2 = the 32-wide tree
-                           searched by a whole warp, one query at a time;
+                           the Morton-cell stop test; 2 = the wide tree searched
+                           by a whole warp (segments: 32 children a node, one
+                           query at a time; triangles: 8 oriented boxes a node,
+                           four queries at a time);
                            3 = routed: after the seed and the outsized elements,
                            a query whose bound excludes both child boxes of the
                            binary root needs no tree search; the others are
-                           searched as in order 2 (for segments, as in order 0
-                           when more than 16 lanes of a warp need one at once);
+                           searched as in order 2 (segments of a tree of at
+                           most 256: as in order 0);
                            -1 = automatic (3; with a Neumann part, 0 while the
                            Dirichlet part has fewer than 128 elements; orders 2
-                           and 3 fall back to 0 without a 32-wide tree) */
+                           and 3 fall back to 0 without a wide tree) */
     int dudn_estimator; /* du/dn at a shell hit from the K nested walks: 0 = backward
                            difference (g(xbar) - mean u(xbar - h n)) / h, Eq.
                            (dudn_fd_estimate); 1 = ball gradient at x_off = xbar - h n:
@@ -149,7 +151,8 @@ typedef struct {
     uint64_t launches;      /* kernels this context has launched since creation */
     float kernel_ms;        /* device time of the last walk kernel (0 if unknown) */
     int blocks;             /* thread blocks of the last walk kernel */
-    uint64_t wide_nodes_visited; /* 32-wide node visits (search orders 2 and 3) */
+    uint64_t wide_nodes_visited; /* wide node visits (search orders 2 and 3), in units
+                                    of 32 child slots (triangles: four nodes) */
 } dwos_run_stats;
 
 /* ---- context ------------------------------------------------------------ */
@@ -266,7 +269,7 @@ dwos_status dwos_set_neumann(dwos_ctx* ctx, const int32_t* flags, int mem);
  * must be finite (DWOS_ERR_INVALID_ARG).  Synchronises. */
 dwos_status dwos_set_neumann_data(dwos_ctx* ctx, const float* h, int mem);
 
-/* Bound on the BVH node fetches (binary nodes, or 32-wide node visits) that one
+/* Bound on the BVH node fetches (binary nodes, or wide node visits) that one
  * distance query of a walk may make; 0 (the default) keeps the trees' own
  * bounds, which a valid tree never reaches.  A query that exceeds the bound
  * keeps the closest element it has found, its walk continues, and the call
@@ -425,8 +428,8 @@ dwos_status dwos_get_vertices(const dwos_ctx* ctx, float* vert, int mem);
 
 /* Sizes of the acceleration structures built by dwos_set_boundary /
  * dwos_set_params: info[0..5] = elements, elements in the binary tree,
- * outsized elements kept out of it, binary inner nodes, 32-wide nodes, levels
- * of the 32-wide tree.  Synchronous (host array). */
+ * outsized elements kept out of it, binary inner nodes, wide nodes (in units of
+ * 32 child slots), levels of the wide tree.  Synchronous (host array). */
 dwos_status dwos_bvh_info(const dwos_ctx* ctx, int32_t* info);
 
 /* Raw per-walk records (n_query x walks_per_point rows, row p*W + w, Philox
