@@ -331,7 +331,7 @@ __global__ void __launch_bounds__(256, STAR ? (DIM == 2 && DATA ? 4 : 3) : DIM =
             // R = max(min(d_D - c, d_sil), eps - c), c = 1e-3 eps the Dirichlet clearance
             const float R = fmaxf(fminf(sqrtf(sd2), fmaf(-1e-3f, P.eps, d)), fmaf(-1e-3f, P.eps, P.eps));
             if (P.f != 0.0f) {   // source: a point of the ball, counted if x sees it
-                const U4 r1 = draw_block(P.seed_lo, P.seed_hi, wid, k_step, (uint32_t)phase, 1u);
+                const U4 r1 = draw_block<!WIDE && !DATA>(P.seed_lo, P.seed_hi, wid, k_step, (uint32_t)phase, 1u);
                 float w[3];
                 sphere_dir<DIM>(r1, w);
                 turn_inward<DIM>(w, on_e, n_on, on2, n2);
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(256, STAR ? (DIM == 2 && DATA ? 4 : 3) : DIM =
                 acc += ds.w;
                 if (!ds.ok) ok2 = false;
             }
-            const U4 r0 = draw_block(P.seed_lo, P.seed_hi, wid, k_step, (uint32_t)phase, 0u);
+            const U4 r0 = draw_block<!WIDE && !DATA>(P.seed_lo, P.seed_hi, wid, k_step, (uint32_t)phase, 0u);
             float om[3];
             sphere_dir<DIM>(r0, om);
             turn_inward<DIM>(om, on_e, n_on, on2, n2);   // on the Neumann part: into the domain
