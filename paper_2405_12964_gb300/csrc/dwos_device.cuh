@@ -801,6 +801,7 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
                 top = ok ? top - 1 - first : max(top - W, 0);
             }
         }
+        __syncwarp();   // every lane has read the stacks (shuffles order no memory): pushes may write them
         // visit
         const bool go = cur >= 0;
         int code = kEmptyChild;
