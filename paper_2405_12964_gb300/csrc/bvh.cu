@@ -580,13 +580,58 @@ __device__ __forceinline__ void leaf_normal(const float4* prims, int p, float* n
     n[2] = u[0] * v[1] - u[1] * v[0];
 }
 
-// The frame of the unit normal n (row 0) and the unit tangent t (row 1).
+// v over its length; false, with v as it was, without a direction.  (Scaled by the largest
+// component first: squares of a small or large mesh's cross products leave FP32's range.)
+__device__ __forceinline__ bool unit(float* v) {
+    const float m = fmaxf(fabsf(v[0]), fmaxf(fabsf(v[1]), fabsf(v[2])));
+    if (!(m > 1e-37f && m < 1e37f)) return false;
+    const float r = 1.0f / m, s[3] = {v[0] * r, v[1] * r, v[2] * r};
+    const float il = rsqrtf(s[0] * s[0] + s[1] * s[1] + s[2] * s[2]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = s[k] * il;
+    return true;
+}
+
+// A unit vector t perpendicular to the unit vector n, from the axis least aligned with n.
+__device__ __forceinline__ void perpendicular(const float* n, float* t) {
+    const float ax = fabsf(n[0]), ay = fabsf(n[1]), az = fabsf(n[2]);
+    if (ax <= ay && ax <= az) { t[0] = 0.0f; t[1] = n[2]; t[2] = -n[1]; }
+    else if (ay <= az) { t[0] = -n[2]; t[1] = 0.0f; t[2] = n[0]; }
+    else { t[0] = n[1]; t[1] = -n[0]; t[2] = 0.0f; }
+    const float il = rsqrtf(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t[k] *= il;
+}
+
+// The frame of the unit normal n (row 0) and the unit tangent t (row 1), perpendicular to
+// each other: a box bounds distances only if its rows are orthonormal.
 __device__ __forceinline__ void frame_rows(const float* n, const float* t, float (*R)[3]) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) { R[0][k] = n[k]; R[1][k] = t[k]; }
     R[2][0] = n[1] * t[2] - n[2] * t[1];
     R[2][1] = n[2] * t[0] - n[0] * t[2];
     R[2][2] = n[0] * t[1] - n[1] * t[0];
+}
+
+// A triangle's frame, from its normal n (any length) and first edge t (R as it was without
+// one).  The thinner the triangle, the more of n is the cross product's rounding, along t as
+// well: what lies along t is taken out (with it left in, boxes of triangles thinner than 1e-3
+// of their length exceeded squared distances by up to |n . t|, beyond what the search allows), and
+// where little else is left any perpendicular serves.
+__device__ __forceinline__ void leaf_frame(float* n, float* t, float (*R)[3]) {
+    if (!unit(t)) return;
+    const bool ok = unit(n);
+    const float d = n[0] * t[0] + n[1] * t[1] + n[2] * t[2];
+    if (ok && d * d < 0.5f) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n[k] = fmaf(-d, t[k], n[k]);
+        const float il = rsqrtf(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) n[k] *= il;
+    } else {
+        perpendicular(t, n);
+    }
+    frame_rows(n, t, R);
 }
 
 // Row r of a frame times (v - o), in the order of the search's box test.
@@ -608,8 +653,8 @@ __device__ __forceinline__ void store_box(float4* wnodes, int slot, const float*
 // The oriented boxes of a 3D tree, one warp per wide node: the node's own box, in its
 // parent's slot, and the boxes of its leaf children and empty slots, one per lane.  A
 // box's frame is the mean normal of the elements under it (each counted along the
-// first one's side; a leaf's own normal and first edge); its extents are taken about
-// its rounded centre, so that only relative rounding is left.
+// first one's side; a leaf's own normal and first edge, made perpendicular); its extents are
+// taken about its rounded centre, so that only relative rounding is left.
 __global__ void oriented_fill_kernel(const float4* nodes, const float4* prims, const int* node_count,
                                      const int* node_first, const int* wcode, const int* wroot, const int* wslot,
                                      int n_wide, float4* wnodes) {
@@ -621,21 +666,12 @@ __global__ void oriented_fill_kernel(const float4* nodes, const float4* prims, c
         float c[3] = {0.0f, 0.0f, 0.0f}, h[3] = {0.0f, 0.0f, 0.0f};
         float R[3][3] = {{1.0f, 0.0f, 0.0f}, {0.0f, 1.0f, 0.0f}, {0.0f, 0.0f, 1.0f}};
         if (my_code < 0) {
-            float v[3][3], n[3], t[3], l2 = 0.0f, t2 = 0.0f;
+            float v[3][3], n[3], t[3];
             for (int a = 0; a < 3; ++a) leaf_vertex(prims, ~my_code, a, v[a]);
             leaf_normal(prims, ~my_code, n);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                t[k] = v[1][k] - v[0][k];
-                l2 = fmaf(n[k], n[k], l2);
-                t2 = fmaf(t[k], t[k], t2);
-            }
-            const float len = sqrtf(l2), tlen = sqrtf(t2);
-            if (len > 0.0f && len < kInf && tlen > 0.0f && tlen < kInf) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) { n[k] /= len; t[k] /= tlen; }
-                frame_rows(n, t, R);
-            }
+            for (int k = 0; k < 3; ++k) t[k] = v[1][k] - v[0][k];
+            leaf_frame(n, t, R);
             float m[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
@@ -688,18 +724,9 @@ __global__ void oriented_fill_kernel(const float4* nodes, const float4* prims, c
         area = warp_fsum(area);
         const float len = sqrtf(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
         // a patch whose normals spread too far keeps the axis-aligned box
-        if (len > 0.7f * area && len > 0.0f && area < kInf) {
+        if (len > 0.7f * area && area < kInf && unit(n)) {
             float t[3], o[3], lo[3], hi[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) n[k] /= len;
-            // the axis least aligned with n gives the tangent
-            const float ax = fabsf(n[0]), ay = fabsf(n[1]), az = fabsf(n[2]);
-            if (ax <= ay && ax <= az) { t[0] = 0.0f; t[1] = n[2]; t[2] = -n[1]; }
-            else if (ay <= az) { t[0] = -n[2]; t[1] = 0.0f; t[2] = n[0]; }
-            else { t[0] = n[1]; t[1] = -n[0]; t[2] = 0.0f; }
-            const float il = rsqrtf(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
-#pragma unroll
-            for (int k = 0; k < 3; ++k) t[k] *= il;
+            perpendicular(n, t);
             frame_rows(n, t, R);
             leaf_vertex(prims, first, 0, o);
 #pragma unroll
