@@ -269,7 +269,8 @@ dwos_status dwos_set_neumann(dwos_ctx* ctx, const int32_t* flags, int mem);
  * must be finite (DWOS_ERR_INVALID_ARG).  Synchronises. */
 dwos_status dwos_set_neumann_data(dwos_ctx* ctx, const float* h, int mem);
 
-/* Bound on the BVH node fetches (binary nodes, or wide node visits) that one
+/* Bound on the BVH node fetches (binary nodes, or wide node visits in the
+ * statistics' units of 32 child slots, for triangles nine nodes at least) that one
  * distance query of a walk may make; 0 (the default) keeps the trees' own
  * bounds, which a valid tree never reaches.  A query that exceeds the bound
  * keeps the closest element it has found, its walk continues, and the call

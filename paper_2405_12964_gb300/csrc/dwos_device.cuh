@@ -669,12 +669,16 @@ __device__ __forceinline__ float obb_dist2(const float* q, const float4* s) {
 // memory (two 32-bit minima: the distance's bits, then the lower leaf index among
 // equals, the order of `closer`), so that groups need not wait for their leaves and
 // several can serve one query.
-// n_nodes counts node visits, n_prims measured leaves.
+// n_nodes counts node visits, n_prims measured leaves.  A caller's bound on a query's
+// visits (budget > 0) counts 32 child slots, four nodes, as a visit, and at least the nine
+// nodes that take the place of one with 32 slots (one and its eight children).  Each group counts
+// its own visits, so the nodes of a query under such a bound do not change hands (a count in
+// shared memory for all groups cost every search 5 %).
 // best2 / best hold each lane's bound on entry (kInf / -1 without one) and
 // the result on exit.  Called by all 32 lanes with the same `need` and each
 // lane's own view (lanes may belong to different problems).  Returns 1 if a
-// group visited more nodes than a query's budget or would overflow its stack
-// (excluded by the stack's size for the tree's depth), which ends its search.
+// query needed more visits than its bound, or than the tree has nodes, or a group would
+// overflow its stack (excluded by the stack's size for the tree's depth), which ends its search.
 __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned need, const float* q_lane, float& best2,
                                                 int& best, SearchScratch* sc, int stk_cap, unsigned& n_nodes,
                                                 unsigned& n_prims) {
@@ -699,7 +703,8 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
     float q[DIM];
 #pragma unroll
     for (int k = 0; k < DIM; ++k) q[k] = 0.0f;
-    int src = 0, top = 0, cur = -1, budget = 0, n_cand = 0;
+    int src = 0, top = 0, cur = -1, n_cand = 0;
+    int budget = 0;                    // twice the visits left, odd without a caller's bound
     const float4* wn = reinterpret_cast<const float4*>(mine.wnodes);
     __syncwarp();
     // measures the listed leaves, one per lane
@@ -748,7 +753,8 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
                     if (take) q[k] = v;
                 }
                 const unsigned long long vp = __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.wnodes), s);
-                const int vb = __shfl_sync(kWarpAll, mine.budget > 0 ? mine.budget : mine.n_wide, s);
+                const int bound = max(min(mine.budget, 1 << 27) * (kWide / W), W + 1);
+                const int vb = __shfl_sync(kWarpAll, mine.budget > 0 ? 2 * bound : 2 * mine.n_wide + 1, s);
                 if (take) {
                     src = s;
                     wn = reinterpret_cast<const float4*>(vp);
@@ -761,7 +767,7 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
                 // no query waits: the k-th idle group takes the top entry of the k-th busy group
                 // that has one, and goes on with that group's query
                 const unsigned heads = idle & kHeads;
-                const unsigned busy = __ballot_sync(kWarpAll, top > 0) & kHeads;
+                const unsigned busy = __ballot_sync(kWarpAll, top > 0 && (budget & 1)) & kHeads;
                 const unsigned under = (1u << gb) - 1u;
                 if (busy) {
                     const int rank = __popc(heads & under);
@@ -814,7 +820,7 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
             for (int k = 0; k < 4; ++k) s[k] = __ldg(f + k * W);
             code = __float_as_int(s[0].w);
             cd = obb_dist2(q, s);
-            if (--budget < 0) { err = 1; code = kEmptyChild; top = 0; }
+            if ((budget -= 2) < 0) { err = 1; code = kEmptyChild; top = 0; if (j == 0) --n_nodes; }
         }
         const bool ok = code != kEmptyChild && within(cd, b2);
         const bool inner = ok && code >= 0;
