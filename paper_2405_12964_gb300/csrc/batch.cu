@@ -255,13 +255,16 @@ dwos_status dwos_batch_create(dwos_batch** out, const dwos_batch_job* jobs, int 
         b->cfg[dim].dim = dim;
         b->cfg[dim].block_size = 256;
         b->cfg[dim].n_sm = b->n_sm;
-        // (two levels to spare: a context may rebuild its tree after the batch was made)
-        for (int ji : ids) b->cfg[dim].wide_depth = std::max(b->cfg[dim].wide_depth, b->jobs[ji].ctx->bvh.wide_depth + 2);
+        for (int ji : ids) b->cfg[dim].wide_depth = std::max(b->cfg[dim].wide_depth, b->jobs[ji].ctx->bvh.wide_depth);
     }
     if (dwos_status s = upload_tables(b)) return bail(s);
-    // the occupancy of the kernel that runs (the search order is set with the tables; asked
+    // The occupancy of the search order's kernel (the order is set with the tables; asked
     // for the per-lane kernel, 3D launches got three blocks per SM: 15.0 ms against 13.9 for
-    // eight problems of up to 20,000 elements, 1.5 M 3D walks)
+    // eight problems of up to 20,000 elements, 1.5 M 3D walks).  Launches of few 3D walks run
+    // a kernel that fits three times, not four; they keep four, which spreads their walks over
+    // fewer lanes of the three resident blocks' warps: two problems, 131,072 walks 2.17 ms
+    // against 2.30 with three (2,048: 0.66 / 0.67; 524,288: 4.93 / 4.95; eight problems,
+    // 131,072: 2.45 / 2.56; 40 problems, 40,960: 2.15 / 2.19).
     for (int dim = 2; dim <= 3; ++dim)
         b->cfg[dim].blocks_per_sm = std::max(1, walk_max_blocks_per_sm(b->cfg[dim]));
     if ((e = cudaEventCreate(&b->ev0)) != cudaSuccess || (e = cudaEventCreate(&b->ev1)) != cudaSuccess)
