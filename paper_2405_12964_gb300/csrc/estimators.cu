@@ -80,12 +80,11 @@ __device__ __forceinline__ void block_sum(double (&v)[NV]) {
     for (int k = 0; k < NV; ++k) v[k] = warp_sum(lane < nw ? sh[k][lane] : 0.0);
 }
 
-// Mean (and standard error) of the first `used` walks of each point's W; with PLAIN also
-// the standard error without the control variate, from the same pass over the records.
+// Mean (and standard error) of the first `used` walks of point p's W, by a block; with PLAIN
+// also the standard error without the control variate, from the same pass over the records.
 template <bool PLAIN>
-__global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int used, double* mean, double* se,
-                                CvView cv, double* se_plain) {
-    const int p = blockIdx.x;
+__device__ __forceinline__ void reduce_point_u(const dwos_record* __restrict__ rec, int p, int W, int used, double* mean,
+                                               double* se, const CvView& cv, double* se_plain) {
     double a[PLAIN ? 4 : 2] = {};
     for (int w = threadIdx.x; w < used; w += blockDim.x) {
         const long long i = (long long)p * W + w;
@@ -106,9 +105,16 @@ __global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int 
     if constexpr (PLAIN) se_plain[p] = std_error(a[3], a[2] / used, used);
 }
 
-// u and the forward-mode derivatives of one point: a cluster of blocks shares the point's
-// walks.  A block takes a range of them 256 at a time: each thread reads one record, adds
-// its u and leaves what the derivatives need (vertices, barycentric weights in FP64, c) in
+template <bool PLAIN>
+__global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int used, double* mean, double* se,
+                                CvView cv, double* se_plain) {
+    reduce_point_u<PLAIN>(rec, blockIdx.x, W, used, mean, se, cv, se_plain);
+}
+
+// u and the forward-mode derivatives of one point.  u: the last blocks (of the highest
+// blockIdx.y), summed as reduce_u does (the same bits).  The derivatives: a cluster of blocks shares the point's
+// walks.  A block takes a range of them 256 at a time: each thread reads one record
+// and leaves what the derivatives need (vertices, barycentric weights in FP64, c) in
 // shared memory; then every thread takes one parameter (column) of every G-th walk.  The
 // FP64 sums are what it costs: packing G = 256 / C walks of C columns to a block keeps the
 // lanes full (17 parameters in a warp of their own left 15 idle), and the cluster spreads a
@@ -128,23 +134,22 @@ __global__ void __launch_bounds__(256) reduce_udot_kernel(const dwos_record* __r
     __shared__ int vid[DIM][256];            // vertices (-1: the walk has no boundary term)
     __shared__ double red[2][256];           // sums of v and v^2 per thread
     __shared__ double part[2][kUdotCols];    // the block's sums per column
-    __shared__ double upart[2];              // and of u
     cg::cluster_group cluster = cg::this_cluster();
     const int S = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int p = blockIdx.x / S, t = threadIdx.x;
+    if (blockIdx.y == gridDim.y - 1) {       // whole clusters
+        if (rank == 0) reduce_point_u<false>(rec, p, W, W, mean, se, CvView{nullptr, nullptr, nullptr, 2, nullptr}, nullptr);
+        return;
+    }
     const int first = blockIdx.y * cols, C = min(cols, N - first), G = 256 / C;
     const int g = t / C, j = first + t % C;
     const int begin = (int)((long long)W * rank / S), end = (int)((long long)W * (rank + 1) / S);
-    double s = 0.0, s2 = 0.0, u[2] = {0.0, 0.0};
+    double s = 0.0, s2 = 0.0;
     for (int base = begin; base < end; base += 256) {
         const int cnt = min(256, end - base);
         __syncthreads();
         if (t < cnt) {
             const dwos_record r = rec[(size_t)p * W + base + t];
-            if (blockIdx.y == 0) {
-                u[0] += (double)r.u;
-                u[1] += (double)r.u * r.u;
-            }
             const float w[3] = {1.0f - r.b1 - r.b2, r.b1, r.b2};
 #pragma unroll
             for (int i = 0; i < DIM; ++i) {
@@ -173,8 +178,7 @@ __global__ void __launch_bounds__(256) reduce_udot_kernel(const dwos_record* __r
     }
     red[0][t] = s;
     red[1][t] = s2;
-    block_sum(u);                            // (a block barrier: red is complete)
-    if (t == 0) { upart[0] = u[0]; upart[1] = u[1]; }
+    __syncthreads();
     if (t < C) {
         for (int k = 1; k < G; ++k) { s += red[0][t + k * C]; s2 += red[1][t + k * C]; }
         part[0][t] = s;
@@ -191,16 +195,6 @@ __global__ void __launch_bounds__(256) reduce_udot_kernel(const dwos_record* __r
             const double m = s / W;
             dmean[(size_t)p * N + j] = m;
             if (dse) dse[(size_t)p * N + j] = std_error(s2, m, W);
-        }
-        if (t == 0 && blockIdx.y == 0) {
-            for (int k = 1; k < S; ++k) {
-                const double* o = cluster.map_shared_rank(&upart[0], k);
-                u[0] += o[0];
-                u[1] += o[1];
-            }
-            const double m = u[0] / W;
-            mean[p] = m;
-            if (se) se[p] = std_error(u[1], m, W);
         }
     }
     cluster.sync();                          // rank 0 has read the others' shared memory
@@ -566,7 +560,7 @@ cudaError_t launch_reduce_udot(const dwos_record* rec, const int* elem, const fl
     // blocks to a point: until the grid has four per SM, each with 64 walks or more
     int S = 1;
     while (S < kUdotCluster && (long long)n_points * ny * S < 4 * 152 && W / (2 * S) >= 64) S *= 2;
-    const dim3 grid((unsigned)n_points * S, ny);
+    const dim3 grid((unsigned)n_points * S, ny + 1);
     return dim == 2 ? launch_cluster(reduce_udot_kernel<2>, grid, 256, S, s, rec, elem, jac, dg, N, W, cols, mean, se,
                                      dmean, dse)
                     : launch_cluster(reduce_udot_kernel<3>, grid, 256, S, s, rec, elem, jac, dg, N, W, cols, mean, se,
