@@ -996,7 +996,7 @@ dwos_status dwos_eval(dwos_ctx* ctx, int n_query, const float* xq, int W, double
         double* dm = mem == DWOS_MEM_DEVICE ? du_mean : ctx->out + 2 * (size_t)n_query;
         double* ds = mem == DWOS_MEM_DEVICE ? du_se : ctx->out + 2 * (size_t)n_query + (size_t)n_query * N;
         CK(launch_reduce_udot(ctx->rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, N, n_query, W, m, se, dm, ds,
-                              ctx->stream), "reduce udot");
+                              ctx->n_sm, ctx->stream), "reduce udot");
     }
     ctx->launches += n_query > 0 ? 1 : 0;
     if (mem == DWOS_MEM_HOST) {
@@ -1712,6 +1712,6 @@ extern "C" dwos_status dwos_eval_static(dwos_ctx* ctx, int n_query, const float*
         CK(launch_reduce_u(d_rec, n_query, W, u_mean, u_se, ctx->stream), "reduce u");
     else
         CK(launch_reduce_udot(d_rec, ctx->elem, ctx->jac, ctx->dg_vert, ctx->dim, ctx->n_param, n_query, W, u_mean,
-                              u_se, du_mean, du_se, ctx->stream), "reduce udot");
+                              u_se, du_mean, du_se, ctx->n_sm, ctx->stream), "reduce udot");
     return DWOS_OK;
 }

@@ -236,7 +236,7 @@ cudaError_t launch_pack_samples(const dwos_record* rec, float4* samples, long lo
 // u and du (reduce_u alone if n_param is 0)
 cudaError_t launch_reduce_udot(const dwos_record* rec, const int* elem, const float* jac, const float* dg,
                                int dim, int n_param, int n_points, int W, double* mean, double* se, double* dmean,
-                               double* dse, cudaStream_t stream);
+                               double* dse, int n_sm, cudaStream_t stream);
 // mode 0: VJP weights w_p / W;  1: U-statistic L2 weights in batches of B;  2: correlated
 // product (umean = mean u of all W walks);  3: uncorrelated product (umean = mean u of the
 // first W/2 walks, weights on the other W/2).

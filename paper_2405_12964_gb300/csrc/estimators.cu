@@ -119,7 +119,9 @@ __global__ void reduce_u_kernel(const dwos_record* __restrict__ rec, int W, int 
 // FP64 sums are what it costs: packing G = 256 / C walks of C columns to a block keeps the
 // lanes full (17 parameters in a warp of their own left 15 idle), and the cluster spreads a
 // few points' walks over the chip.  64 points x 1024 walks, 17 parameters: 104 us as one
-// block per point and a kernel of its own for u, 30 us now.
+// block per point and a kernel of its own for u, 27.5 us now.  The G sums of a column are
+// halved in turn (added by one thread each, one column cost 25 us of a chain of 255
+// FP64 sums: 1 x 4096 walks, 1 parameter 26.5 -> 9.5 us, 700 x 64 38.4 -> 18.3).
 constexpr int kUdotCols = 128;      // columns a block takes at most (blockIdx.y: chunks of them)
 constexpr int kUdotCluster = 8;     // blocks of a point's cluster at most
 
@@ -176,11 +178,14 @@ __global__ void __launch_bounds__(256) reduce_udot_kernel(const dwos_record* __r
                 s2 += v * v;
             }
     }
-    red[0][t] = s;
-    red[1][t] = s2;
-    __syncthreads();
+    for (int n = G; n > 1;) {                // the G sums of each column, halved in turn
+        const int half = (n + 1) / 2;
+        if (g >= half && g < n) { red[0][t] = s; red[1][t] = s2; }
+        __syncthreads();
+        if (g < n - half) { s += red[0][t + half * C]; s2 += red[1][t + half * C]; }
+        n = half;
+    }
     if (t < C) {
-        for (int k = 1; k < G; ++k) { s += red[0][t + k * C]; s2 += red[1][t + k * C]; }
         part[0][t] = s;
         part[1][t] = s2;
     }
@@ -553,13 +558,18 @@ cudaError_t launch_pack_samples(const dwos_record* rec, float4* samples, long lo
 
 cudaError_t launch_reduce_udot(const dwos_record* rec, const int* elem, const float* jac, const float* dg, int dim,
                                int N, int n_points, int W, double* mean, double* se, double* dmean, double* dse,
-                               cudaStream_t s) {
+                               int n_sm, cudaStream_t s) {
     if (n_points <= 0) return cudaSuccess;
     if (N <= 0) return launch_reduce_u(rec, n_points, W, mean, se, s);
-    const int ny = (N + kUdotCols - 1) / kUdotCols, cols = (N + ny - 1) / ny;
-    // blocks to a point: until the grid has four per SM, each with 64 walks or more
+    // until the grid has four blocks per SM: chunks of fewer columns, 32 at least (128 columns of
+    // 1 x 64 walks in one block 18.9 us, in four 8.5; 64 x 1024 128 -> 110; 700 points: no split), then
+    // blocks to a point, each with 64 walks or more
+    int ny = (N + kUdotCols - 1) / kUdotCols;
+    while (ny * 32 < N && (long long)n_points * ny < 4 * n_sm) ny *= 2;
+    const int cols = (N + ny - 1) / ny;
+    ny = (N + cols - 1) / cols;
     int S = 1;
-    while (S < kUdotCluster && (long long)n_points * ny * S < 4 * 152 && W / (2 * S) >= 64) S *= 2;
+    while (S < kUdotCluster && (long long)n_points * ny * S < 4 * n_sm && W / (2 * S) >= 64) S *= 2;
     const dim3 grid((unsigned)n_points * S, ny + 1);
     return dim == 2 ? launch_cluster(reduce_udot_kernel<2>, grid, 256, S, s, rec, elem, jac, dg, N, W, cols, mean, se,
                                      dmean, dse)
