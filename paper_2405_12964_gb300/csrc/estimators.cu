@@ -412,10 +412,10 @@ __global__ void gemv_kernel(const float* __restrict__ jac, const float* __restri
 
 // mean[p] * scale is the point's mean (scale 1 / W for per-point sums); it is
 // also written to mean_out when given.  One cluster: FP64 arithmetic bounds the sum, so
-// many points are shared by its blocks (16384 points: 43 us in one block, 10 us in eight),
-// and rank 0 adds the blocks' sums in order.
+// many points are shared by its blocks, and rank 0 adds the blocks' sums in order (one block /
+// eight, us: 512 points 2.6 / 3.6, 1024 3.4 / 3.4, 2048 5.0 / 3.7, 16384 26 / 6.6).
 constexpr int kLossCluster = 8;
-constexpr int kLossSplit = 2048;    // points from which a cluster of blocks is worth its barriers
+constexpr int kLossSplit = 1024;    // points from which a cluster of blocks is worth its barriers
 
 __global__ void __launch_bounds__(256) loss_kernel(const double* mean, const float* uref, const float* pweight, int n,
                                                    double* loss, double scale, double* mean_out) {
@@ -430,12 +430,12 @@ __global__ void __launch_bounds__(256) loss_kernel(const double* mean, const flo
     }
     block_sum(s);
     if (threadIdx.x == 0) total = s[0];
-    cluster.sync();
+    if (gridDim.x > 1) cluster.sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         for (int k = 1; k < (int)gridDim.x; ++k) s[0] += *cluster.map_shared_rank(&total, k);
         *loss = s[0];
     }
-    cluster.sync();                 // the first block has read the others' sums
+    if (gridDim.x > 1) cluster.sync();     // the first block has read the others' sums
 }
 
 // One launch with clusters of `size` blocks along x.
