@@ -2,15 +2,16 @@
 // -> 4 x 64 tanh -> 8 linear outputs (0: u, 1: du/dn), trained and evaluated
 // on the 5th-generation tensor cores.
 //
-// One persistent kernel (512 threads, one CTA per SM) walks over tiles of 128
-// samples; sample row r is TMEM lane r, and threads r, r + 128, r + 256 and r + 384
-// share it (warps w, w + 4, ... reach the same TMEM lane quarter): each takes 16 of the
+// One persistent kernel (one CTA per SM; 512 threads in training, 256 in evaluation) walks
+// over tiles of 128 samples; sample row r is TMEM lane r, and threads r, r + 128, ...
+// share it (warps w, w + 4, ... reach the same TMEM lane quarter): each takes 16 (32) of the
 // row's 64 columns in the epilogues between the products.  The ten products of a tile
 // are a chain (each operand is the last product's epilogue), so a CTA's time is the
 // chain's latency: four threads to a row instead of two halve the issue time of the
 // tanh epilogues, each link has one block barrier, and the weight gradients of a layer
 // run while the threads work on the next layer's deltas (two delta tiles in turn):
-// 65,536 rows 55 us with two threads to a row and two barriers a link, 45 us now.
+// 65,536 rows 50.9 us with two threads to a row and two barriers a link, 42.5 so, 36.6 with
+// the layers unrolled (evaluation 32.9 / 35.9 / 32.5).
 // Operands
 // live in shared memory as BF16 in the canonical no-swizzle core-matrix
 // layout (8 rows x 16 bytes per 128-byte core matrix), the products are
@@ -44,7 +45,6 @@ constexpr int OUT = 8;           // output width
 constexpr int OUTP = 16;         // output rows padded for the N = 16 product
 constexpr int NP = DWOS_MLP_NPARAM;
 constexpr int TILE = 128;        // samples per tile (the MMA's M)
-constexpr int THREADS = 512;          // four threads per sample row
 // offsets of W_l and b_l (l = 1..5) in the flat parameter vector
 __host__ __device__ constexpr int off_w(int l) { return l == 1 ? 0 : 1088 + (l - 2) * 4160; }
 __host__ __device__ constexpr int off_b(int l) { return l == 1 ? 1024 : (l == 5 ? 14080 : 1088 + (l - 2) * 4160 + 4096); }
@@ -78,7 +78,6 @@ struct __align__(1024) Smem {
     float bias[4 * H + OUT];
     unsigned long long bar_load, bar_mma;
     uint32_t tmem_base;
-    int fail;
 };
 
 // TMEM columns (512 allocated)
@@ -198,11 +197,16 @@ __device__ __forceinline__ void feats(float x, float y, float* f) {
 
 enum Mode { kTrain = 0, kEval = 1 };
 
+// Threads to a sample row: four in training; two in evaluation, which has no weight gradients
+// to run beside the epilogues (262,144 rows: 107.9 us with four, 106.9 with two).
+constexpr int row_threads(int mode) { return mode == kTrain ? 4 : 2; }
+constexpr int threads(int mode) { return TILE * row_threads(mode); }
+
 // mode kTrain: masked-MSE loss (sums of this CTA's four warps of rows at loss + 4 *
 // blockIdx.x) and the CTA's gradient partial (NP floats at part + blockIdx.x * NP).
 // mode kEval: u, d u / d (x, y) and du/dn per sample.
 template <int MODE>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(threads(MODE), 1)
     mlp_kernel(const WImage* __restrict__ wimg, const float* __restrict__ params, int n,
                const float* __restrict__ x, const float* __restrict__ target, const float* __restrict__ mask,
                float* __restrict__ part, double* __restrict__ loss, float* __restrict__ u_out,
@@ -211,13 +215,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     Smem& S = *reinterpret_cast<Smem*>(raw);
     const int tid = threadIdx.x;
     const int r = tid & (TILE - 1);            // sample row and TMEM lane
-    const int q16 = tid >> 7;                  // which 16 of the row's columns this thread takes
+    constexpr int Q = row_threads(MODE);       // columns 16 c .. 16 c + 15 of a row, c = q, q + Q, ... < 4, are this thread's
+    const int q = tid / TILE;
     const int warp = tid >> 5;
     const uint32_t bar_load = smem_u32(&S.bar_load), bar_mma = smem_u32(&S.bar_mma);
     if (tid == 0) {
         bar_init(bar_load, 1);
         bar_init(bar_mma, 1);
-        S.fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         bar_expect_tx(bar_load, sizeof(WImage));
         bulk_g2s(smem_u32(&S.w), wimg, sizeof(WImage), bar_load);
@@ -229,21 +233,23 @@ __global__ void __launch_bounds__(THREADS, 1)
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     // constants: biases; zero the columns of the tiles that no tile overwrites
-    for (int i = tid; i < 4 * H + OUT; i += THREADS)
+    for (int i = tid; i < 4 * H + OUT; i += threads(MODE))
         S.bias[i] = params[i < 4 * H ? off_b(1 + i / H) + i % H : off_b(5) + (i - 4 * H)];
     {
         const float z[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         const float one[8] = {1, 0, 0, 0, 0, 0, 0, 0};
-        if (q16 == 0) {
-            put8(S.a0, C0, r, 1, z);
-            put8(S.a0, C0, r, 2, one);
-            put8(S.a0, C0, r, 3, z);
-        }
-        put8(S.a[q16], CA, r, 8, one);
-        put8(S.a[q16], CA, r, 9, z);
-        for (int cc = q16; cc < CD / 8; cc += 4) {
-            put8(S.d[0], CD, r, cc, z);
-            put8(S.d[1], CD, r, cc, z);
+        if (q == 0) put8(S.a0, C0, r, 1, z);
+        if (MODE == kTrain) {        // read by the weight gradients alone
+            if (q == 0) {
+                put8(S.a0, C0, r, 2, one);
+                put8(S.a0, C0, r, 3, z);
+            }
+            put8(S.a[q], CA, r, 8, one);
+            put8(S.a[q], CA, r, 9, z);
+            for (int cc = q; cc < CD / 8; cc += Q) {
+                put8(S.d[0], CD, r, cc, z);
+                put8(S.d[1], CD, r, cc, z);
+            }
         }
     }
     fence_before();
@@ -280,7 +286,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     auto load_sample = [&](int tile) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) f[i] = 0.0f;
-        if (q16 != 0 || tile >= n_tiles) return;
+        if (q != 0 || tile >= n_tiles) return;
         const int s = tile * TILE + r;
         if (s >= n) return;
         px = x[2 * s];
@@ -297,10 +303,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++tiles_done) {
         const int s = tile * TILE + r;
         const bool valid = s < n;
-        if (q16 == 0) put8(S.a0, C0, r, 0, f);
+        if (q == 0) put8(S.a0, C0, r, 0, f);
         publish();
         if (!ok) break;
-        // ---- forward: four tanh layers
+        // ---- forward: four tanh layers (unrolled, here and below: the operands' descriptors are then
+        // constants and not computed in the chain)
+#pragma unroll
         for (int l = 1; l <= 4; ++l) {
             const __nv_bfloat16* A = l == 1 ? S.a0 : S.a[l - 2];
             const int CAin = l == 1 ? C0 : CA;
@@ -311,12 +319,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                 mma_commit(bar_mma);
             }
             wait_mma();
-            float v[16];
-            tmem_ld16(lane_addr + T_SCR + 16 * q16, v);
+            for (int c = q; c < H / 16; c += Q) {
+                float v[16];
+                tmem_ld16(lane_addr + T_SCR + 16 * c, v);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = tanhf(v[i] + S.bias[(l - 1) * H + 16 * q16 + i]);
-            put8(S.a[l - 1], CA, r, 2 * q16, v);
-            put8(S.a[l - 1], CA, r, 2 * q16 + 1, v + 8);
+                for (int i = 0; i < 16; ++i) v[i] = tanhf(v[i] + S.bias[(l - 1) * H + 16 * c + i]);
+                put8(S.a[l - 1], CA, r, 2 * c, v);
+                put8(S.a[l - 1], CA, r, 2 * c + 1, v + 8);
+            }
             publish();
             if (!ok) break;
         }
@@ -329,7 +339,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             mma_commit(bar_mma);
         }
         wait_mma();
-        if (q16 == 0) {
+        if (q == 0) {
             float o[16];
             tmem_ld16(lane_addr + T_SCR, o);
             float d5[16];
@@ -359,6 +369,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ---- backward: the deltas, and weight gradients (training).  Layer l's weight
         // gradient is issued after its delta product was committed: the wait on that product
         // covers layer l + 1's weight gradient, which read the delta tile written next.
+#pragma unroll
         for (int l = 5; l >= 1; --l) {
             const __nv_bfloat16* Ain = l == 1 ? S.a0 : S.a[l - 2];
             const __nv_bfloat16* D = S.d[l & 1];
@@ -384,20 +395,22 @@ __global__ void __launch_bounds__(THREADS, 1)
             wait_mma();
             if (l > 1) {
                 // delta_{l-1} = (delta_l W_l) * (1 - a_{l-1}^2), a as stored (BF16)
-                float v[16], a[16];
-                tmem_ld16(lane_addr + T_SCR + 16 * q16, v);
-                get8(S.a[l - 2], CA, r, 2 * q16, a);
-                get8(S.a[l - 2], CA, r, 2 * q16 + 1, a + 8);
+                for (int c = q; c < H / 16; c += Q) {
+                    float v[16], a[16];
+                    tmem_ld16(lane_addr + T_SCR + 16 * c, v);
+                    get8(S.a[l - 2], CA, r, 2 * c, a);
+                    get8(S.a[l - 2], CA, r, 2 * c + 1, a + 8);
 #pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] *= 1.0f - a[i] * a[i];
-                put8(S.d[(l - 1) & 1], CD, r, 2 * q16, v);
-                put8(S.d[(l - 1) & 1], CD, r, 2 * q16 + 1, v + 8);
+                    for (int i = 0; i < 16; ++i) v[i] *= 1.0f - a[i] * a[i];
+                    put8(S.d[(l - 1) & 1], CD, r, 2 * c, v);
+                    put8(S.d[(l - 1) & 1], CD, r, 2 * c + 1, v + 8);
+                }
                 publish();
                 if (!ok) break;
             } else if (MODE == kEval) {
                 float df[16];
-                if (q16 == 0) tmem_ld16(lane_addr + T_SCR, df);       // d u / d features
-                if (q16 == 0 && valid && g_out) {
+                if (q == 0) tmem_ld16(lane_addr + T_SCR, df);       // d u / d features
+                if (q == 0 && valid && g_out) {
                     const float c0 = 3.14159265358979f * cospif(px), c1 = 3.14159265358979f * cospif(py);
                     const float c01 = 3.14159265358979f * cospif(px + py);
                     g_out[2 * s] = df[0] + df[2] * c0 + df[4] * c01;
@@ -414,13 +427,13 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     if (MODE == kTrain && ok) {
         for (int off = 16; off > 0; off >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, off);
-        if ((tid & 31) == 0 && q16 == 0) loss[4 * blockIdx.x + warp] = (double)loss_acc * (double)inv_n;
+        if ((tid & 31) == 0 && q == 0) loss[4 * blockIdx.x + warp] = (double)loss_acc * (double)inv_n;
         // the CTA's weight and bias gradients: rows (outputs) are TMEM lanes 0..63
         float* P = part + (size_t)blockIdx.x * NP;
         for (int l = 1; l <= 5; ++l) {
             const int outs = l == 5 ? OUT : H, ins = l == 1 ? IN : H;
             const int ncol = l == 1 ? C0 : CA;
-            for (int c16 = q16; c16 < ncol / 16; c16 += 4) {
+            for (int c16 = q; c16 < ncol / 16; c16 += Q) {
                 float v[16];
                 __syncwarp();
                 tmem_ld16(lane_addr + t_dw(l) + 16 * c16, v);     // warp-wide: every warp loads
@@ -606,7 +619,7 @@ dwos_status check_err(dwos_mlp* mlp) {
 
 // The training kernel: gradient and loss partials of the grid's CTAs.
 dwos_status launch_train(dwos_mlp* mlp, int n, const float* x, const float* t, const float* mk) {
-    mlp_kernel<kTrain><<<grid_for(mlp, n), THREADS, sizeof(Smem), mlp->stream>>>(
+    mlp_kernel<kTrain><<<grid_for(mlp, n), threads(kTrain), sizeof(Smem), mlp->stream>>>(
         mlp->w, mlp->p, n, x, t, mk, mlp->part, mlp->loss_part, nullptr, nullptr, nullptr, mlp->dflag);
     MK(cudaGetLastError(), "train kernel");
     return DWOS_OK;
@@ -751,7 +764,7 @@ dwos_status dwos_mlp_eval(dwos_mlp* mlp, int n, const float* x, float* u, float*
         dg = du + n;
         dq = dg + 2 * (size_t)n;
     }
-    mlp_kernel<kEval><<<grid_for(mlp, n), THREADS, sizeof(Smem), mlp->stream>>>(
+    mlp_kernel<kEval><<<grid_for(mlp, n), threads(kEval), sizeof(Smem), mlp->stream>>>(
         mlp->w, mlp->p, n, d[0], nullptr, nullptr, nullptr, nullptr, du, dg, dq, mlp->dflag);
     MK(cudaGetLastError(), "eval");
     if (mem == DWOS_MEM_HOST) {
