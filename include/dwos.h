@@ -95,7 +95,7 @@ typedef struct {
                            a query whose bound excludes both child boxes of the
                            binary root needs no tree search; the others are
                            searched as in order 2 (segments of a tree of at
-                           most 256: as in order 0);
+                           most 256, as in order 0 when many lanes need it);
                            -1 = automatic (3; with a Neumann part, 0 while the
                            Dirichlet part has fewer than 128 elements; orders 2
                            and 3 fall back to 0 without a wide tree) */

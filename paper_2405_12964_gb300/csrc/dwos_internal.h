@@ -66,7 +66,7 @@ struct DevProblem {
     float r_max;                // element radius bound for the cell test
     int traversal;              // 0 root-down, 1 climb from the hint leaf, 2 by the warp over the wide tree,
                                 // 3 routed: no tree search if the binary root's child boxes are outside the
-                                // bound, else as 2 (2D: per lane for small trees)
+                                // bound, else as 2 (2D: per lane for small trees that many lanes need)
     const float* wnodes;        // wide tree (2D 32-wide, 3D 8-wide nodes), root first
     int n_wide;                 // its node count
     int data_kind;              // 0 mapped, 1 field

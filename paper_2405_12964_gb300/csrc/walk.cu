@@ -29,11 +29,14 @@ constexpr unsigned kFull = 0xffffffffu;
 // Search order 3 routes each query by the binary root's two child boxes: most
 // queries (closer to an outsized element, or to their seed, than to any tree
 // box) need no tree search at all; the few that do are searched by the whole
-// warp over the wide tree.  Trees of at most kLaneTreeMax segments are searched one
-// query per lane, over the binary tree (128 segments: 0.34 ms against 0.42 ms by groups
-// of lanes); for larger ones, and for triangles, that never pays (2.1 M walks around a
-// 4096-segment star, half of whose queries need the tree: 7.5 ms when steps with more
-// than 16 such lanes went one per lane, 6.4 ms without).
+// warp over the wide tree.  Small trees of segments are searched one query per lane, over
+// the binary tree, when many lanes of the warp need it: the lanes' searches run side by side, the
+// warp's one after the other.  The line, n segments < 32 (lanes - 1) and n <= kLaneTreeMax:
+// around a star, where few lanes need the tree (524,288 walks, n = 64 / 96 / 256, us): this
+// 355 / 248 / 255, never per lane 996 / 246 / 246, always 366 / 319 / 393, with more than 16 lanes 415 /
+// 245 / 255; in a disk, where all do (262,144 walks, n = 64 / 128 / 256): 443 / 593 / 802, never 680 /
+// 758 / 871, always 492 / 649 / 875.  Above 256 the warp's search always wins (disk, n = 320: 798 against 998;
+// 4096: 1860 / 5660), and for triangles too.
 constexpr int kLaneTreeMax = 256;
 
 template <int DIM>
@@ -271,7 +274,7 @@ __global__ void __launch_bounds__(256, STAR ? (DIM == 2 && DATA ? 4 : 3) : DIM =
                 }
                 need = __ballot_sync(kFull, desc);
                 if (DIM == 2) {
-                    lane_search = desc && Pw.n_tree <= kLaneTreeMax;
+                    lane_search = desc && Pw.n_tree <= kLaneTreeMax && Pw.n_tree < 32 * (__popc(need) - 1);
                     need = __ballot_sync(kFull, desc && !lane_search);
                 }
             }
