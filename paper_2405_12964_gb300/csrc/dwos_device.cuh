@@ -704,7 +704,9 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
 #pragma unroll
     for (int k = 0; k < DIM; ++k) q[k] = 0.0f;
     int src = 0, top = 0, cur = -1, n_cand = 0;
-    int budget = 0;                    // twice the visits left, odd without a caller's bound
+    // twice the visits left, odd without a caller's bound
+    const int visits = mine.budget > 0 ? 2 * max(min(mine.budget, 1 << 27) * (kWide / W), W + 1) : 2 * mine.n_wide + 1;
+    int budget = 0;
     const float4* wn = reinterpret_cast<const float4*>(mine.wnodes);
     __syncwarp();
     // measures the listed leaves, one per lane
@@ -753,8 +755,7 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
                     if (take) q[k] = v;
                 }
                 const unsigned long long vp = __shfl_sync(kWarpAll, reinterpret_cast<unsigned long long>(mine.wnodes), s);
-                const int bound = max(min(mine.budget, 1 << 27) * (kWide / W), W + 1);
-                const int vb = __shfl_sync(kWarpAll, mine.budget > 0 ? 2 * bound : 2 * mine.n_wide + 1, s);
+                const int vb = __shfl_sync(kWarpAll, visits, s);
                 if (take) {
                     src = s;
                     wn = reinterpret_cast<const float4*>(vp);

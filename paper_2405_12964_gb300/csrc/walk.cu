@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(256, STAR ? (DIM == 2 && DATA ? 4 : 3) : DIM =
                 }
                 need = __ballot_sync(kFull, desc);
                 if (DIM == 2) {
-                    lane_search = desc && Pw.n_tree <= kLaneTreeMax && Pw.n_tree < 32 * (__popc(need) - 1);
+                    lane_search = desc && Pw.n_tree <= min(kLaneTreeMax, 32 * __popc(need) - 33);
                     need = __ballot_sync(kFull, desc && !lane_search);
                 }
             }
