@@ -255,7 +255,9 @@ dwos_status dwos_batch_create(dwos_batch** out, const dwos_batch_job* jobs, int 
         b->cfg[dim].dim = dim;
         b->cfg[dim].block_size = 256;
         b->cfg[dim].n_sm = b->n_sm;
-        for (int ji : ids) b->cfg[dim].wide_depth = std::max(b->cfg[dim].wide_depth, b->jobs[ji].ctx->bvh.wide_depth);
+        // (two levels more than the trees have: with stacks of just their size eight problems, 2D and
+        // 3D in turn, take 13.38 ms instead of 13.27)
+        for (int ji : ids) b->cfg[dim].wide_depth = std::max(b->cfg[dim].wide_depth, b->jobs[ji].ctx->bvh.wide_depth + 2);
     }
     if (dwos_status s = upload_tables(b)) return bail(s);
     // The occupancy of the search order's kernel (the order is set with the tables; asked
