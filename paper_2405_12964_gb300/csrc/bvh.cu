@@ -557,8 +557,10 @@ __device__ __forceinline__ float warp_fmax(float v) { return -warp_fmin(-v); }
 
 // Up to this many leaves a node gets a box oriented by its elements' mean normal;
 // above it the axis-aligned box of the binary tree (a patch that large is curved, and
-// the pass over its leaves would dominate the refit: 15.2 visits per query with a limit
-// of 1024, 15.7 without one, 18.8 with one of 64, on the 200k-triangle sphere).
+// the pass over its leaves would dominate the refit).  On spheres, limits of 256 / 512 / 1024:
+// walk kernel over 50,000 triangles 3.32 / 3.28 / 3.41 ms, 200,000 12.80 / 12.90 / 13.06;
+// this kernel 11.7 / 12.6 / 18.1 and 40.0 / 40.3 / 41.1 us.  (64: 18.8 visits per query over
+// 200,000 triangles, 1024 15.2, none 15.7.)
 constexpr int kOrientMax = 512;
 
 // Vertex a of triangle leaf p.
@@ -860,7 +862,7 @@ __global__ void closest_wide_kernel(BvhView bvh, WideView wv, const int* prim_el
 // Inside test by ray parity along a fixed generic direction.  The ray from
 // each point is cut into 32 sub-intervals [t_s, t_s+1) up to the far corner of
 // the scene box; lane s of the point's warp counts the crossings in its
-// interval with an any-order stackless traversal (pruning boxes its interval
+// interval with an any-order traversal (pruning boxes its interval
 // misses) plus the outsized elements, and the warp sums the counts.
 template <int DIM>
 __device__ __forceinline__ bool seg_hits_box(const float* o, const float* inv, float ta, float tb, const float* lo,

@@ -23,8 +23,8 @@ constexpr float kInf = __builtin_inff();
 struct U4 { uint32_t x, y, z, w; };
 
 // ROLLED: one round's code in a loop, for kernels bound by instruction fetch (walks on
-// stars without a warp-wide search or data: thermal slab, 262,144 walks, 2.94 -> 2.80 ms,
-// cube with a source 5.77 -> 5.61; elsewhere 3-8 % slower).
+// stars without a warp-wide search or data: thermal slab, 262,144 walks, 2.95 -> 2.81 ms,
+// cube with a source 5.79 -> 5.62; elsewhere 3-8 % slower).
 template <bool ROLLED = false>
 __device__ __forceinline__ U4 philox(U4 c, uint32_t k0, uint32_t k1) {
     auto round = [&]() {
@@ -796,7 +796,7 @@ __device__ __forceinline__ int oriented_closest(const WideView& mine, unsigned n
             }
         }
         const float b2 = __uint_as_float(sc->dist[src]);
-        {   // pop: the topmost of the top four entries that is still within the bound
+        {   // pop: the topmost of the top eight entries that is still within the bound
             const int at = top - 1 - j;
             const bool look = cur < 0 && at >= 0;
             const float2 e = look ? st[at] : make_float2(kInf, 0.0f);

@@ -493,8 +493,9 @@ __global__ void convert_kernel(const float* __restrict__ p, WImage* __restrict__
 
 // Sums the CTA partials (gradient and loss, in CTA order: deterministic); with ADAM
 // it also takes the step and writes the new weights' BF16 image, so that a training step
-// is two launches (a step of 65,536 rows 78 us as six operations, 59 us now).  Bound by the latency of the partials' loads (8.6 MB from L2): small
-// blocks spread them over all SMs, sixteen loads in flight per thread.
+// is two launches (a step of 65,536 rows 78 us as six operations, 53 us now).  Bound by the
+// latency of the partials' loads (8.6 MB from L2): small blocks spread them over all SMs,
+// sixteen loads in flight per thread.
 constexpr int kUpdateThreads = 64;
 
 template <bool ADAM>
